@@ -308,6 +308,9 @@ int batch_graph(csc_handle_t h, const PhaseParams &pp, const PhaseConfig &cfg, i
     append_bytes(key, cfg.block);
     append_bytes(key, cfg.smem);
     append_bytes(key, cfg.tile_in_smem);
+    append_bytes(key, cfg.reg_nq);
+    append_bytes(key, cfg.reg_ns);
+    append_bytes(key, cfg.reg_cb);
     append_bytes(key, S);
     append_bytes(key, resident);
     append_bytes(key, h->c);

@@ -207,9 +207,12 @@ struct PhaseParams {
 };
 
 struct PhaseConfig {
-    int block;
-    size_t smem;
-    bool tile_in_smem;
+    int block = 0;
+    size_t smem = 0;
+    bool tile_in_smem = false;
+    // the register form (kernel_phase_reg.cu) when reg_nq > 0: float4 groups of
+    // atoms per thread, columns per thread, threads per group of atoms
+    int reg_nq = 0, reg_ns = 0, reg_cb = 0;
 };
 
 // w_max: widest segment of the plan; threads_per_segment: 32 = one warp per

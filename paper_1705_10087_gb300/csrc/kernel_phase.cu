@@ -41,6 +41,7 @@
 #include <type_traits>
 
 #include "csc_internal.cuh"
+#include "phase_reg.cuh"
 
 namespace csc {
 
@@ -949,13 +950,19 @@ PhaseConfig phase_config(int K, int L, int wmax, int threads_per_segment)
         cfg.smem = Layout(K, wmax, true, true).total;
         return cfg;
     }
+    if (phase_reg_config(K, L, wmax, &cfg))
+        return cfg;
     // An update touches the 2L-1 window columns: with at least that many threads
     // each of them goes to its own thread, however wide the segment; more threads
     // would idle in the update and only cost registers and occupancy.  The block
     // is a power of two (128, 512 or 1024) so that ownership is a mask.
     cfg.block = 2 * L - 1 <= 128 ? 128 : (2 * L - 1 <= 512 ? 512 : 1024);
     const bool vec = vec_layout(K, cfg.block);
-    cfg.tile_in_smem = Layout(K, (int)wmax, true, vec).total <= (size_t)kMaxSmem;
+    // (the compile-time-K kernels that phase_reg_config always takes over where
+    // the tile fits exist in their in-place form only)
+    const bool in_place = vec && !(K == 64 && cfg.block == 512);
+    cfg.tile_in_smem =
+        !in_place && Layout(K, (int)wmax, true, vec).total <= (size_t)kMaxSmem;
     cfg.smem = Layout(K, (int)wmax, cfg.tile_in_smem, vec).total;
     return cfg;
 }
@@ -969,17 +976,19 @@ cudaError_t dispatch(const PhaseConfig &cfg, int K, F &&f)
     // one warp per segment (phase_config checked K == 25 and the window)
     if (cfg.block == 32)
         return f(Sel<true, 32, 25>::fn());
-    // the workloads' atom counts (25 and 64) are compiled with K fixed
+    // the workloads' atom counts (25 and 64) are compiled with K fixed (their
+    // staged form only where phase_reg_config refuses what would fit: K = 64 with
+    // windows of more than 255 columns)
     if (cfg.block == 128) {
         if (K == 25)
-            return cfg.tile_in_smem ? f(Sel<true, 128, 25>::fn()) : f(Sel<false, 128, 25>::fn());
+            return f(Sel<false, 128, 25>::fn());
         if (K == 64)
-            return cfg.tile_in_smem ? f(Sel<true, 128, 64>::fn()) : f(Sel<false, 128, 64>::fn());
+            return f(Sel<false, 128, 64>::fn());
         return cfg.tile_in_smem ? f(Sel<true, 128, 0>::fn()) : f(Sel<false, 128, 0>::fn());
     }
     if (cfg.block == 512) {
         if (K == 25)
-            return cfg.tile_in_smem ? f(Sel<true, 512, 25>::fn()) : f(Sel<false, 512, 25>::fn());
+            return f(Sel<false, 512, 25>::fn());
         if (K == 64)
             return cfg.tile_in_smem ? f(Sel<true, 512, 64>::fn()) : f(Sel<false, 512, 64>::fn());
         return cfg.tile_in_smem ? f(Sel<true, 512, 0>::fn()) : f(Sel<false, 512, 0>::fn());
@@ -1025,6 +1034,8 @@ cudaError_t launch_phase(const PhaseParams &pp, const PhaseConfig &cfg, int acti
 {
     if (active == 0)
         return cudaSuccess;
+    if (cfg.reg_nq > 0)
+        return launch_phase_reg(pp, cfg, active, false, s);
     cudaError_t e = check(pp, cfg);
     if (e != cudaSuccess)
         return e;
@@ -1046,6 +1057,8 @@ int phase_resident_blocks(const PhaseConfig &cfg, int K)
     int per_sm = 1, dev = 0, nsm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (cfg.reg_nq > 0)
+        return nsm * std::max(1, phase_reg_blocks_per_sm(cfg));
     dispatch<Drain>(cfg, K, [&](auto kern) -> cudaError_t {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, cfg.block, cfg.smem);
@@ -1060,7 +1073,7 @@ cudaError_t launch_phase_drain(const PhaseParams &pp, const PhaseConfig &cfg, in
 {
     if (active == 0)
         return cudaSuccess;
-    cudaError_t e = check(pp, cfg);
+    cudaError_t e = cfg.reg_nq > 0 ? cudaSuccess : check(pp, cfg);
     if (e != cudaSuccess)
         return e;
     // queue length and head (two adjacent ints) start at 0
@@ -1074,6 +1087,8 @@ cudaError_t launch_phase_drain(const PhaseParams &pp, const PhaseConfig &cfg, in
     if (e != cudaSuccess)
         return e;
     const int grid = resident < active ? resident : active;
+    if (cfg.reg_nq > 0)
+        return launch_phase_reg(pp, cfg, grid, true, s);
     e = dispatch<Drain>(cfg, pp.K, [&](auto kern) -> cudaError_t {
         cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)cfg.smem);
