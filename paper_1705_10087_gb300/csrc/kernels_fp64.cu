@@ -139,30 +139,15 @@ __global__ void __launch_bounds__(256)
         lists.count[b] = base;
 }
 
-// The refreshed r of coordinate (k, t) of problem sd from beta0 and the
-// double-float sum (ah, al) of its S Z terms, and its share of the report:
-// drift |r_old - r|, zero_excess, nonzero_gap, max |Delta Z| and the
-// coord_step change on the float state (marking its segment dirty when that
-// change is >= tol_mark, or the problem's tol when tol_mark < 0).
-// (b0, rold, z, n: beta0, r, Z of the coordinate and ||D_k||^2, already loaded)
-__device__ __forceinline__ void resync_finish_v(const SigDesc &sd, int64_t ix, int64_t t,
-                                                float b0, float rold, float z, float n, float rn,
-                                                float *__restrict__ rr, float ah, float al,
-                                                float lam, int write_r,
-                                                unsigned char *__restrict__ dirty, float tol_mark,
-                                                float &drift, float &zex, float &nzg, float &all,
-                                                float &dz32)
+// The report of coordinate t of problem sd with refreshed value r32 (rt: the state
+// that is tested, r32 once written): its share of zero_excess, nonzero_gap, max
+// |Delta Z| and the coord_step change on the float state (marking its segment
+// dirty when that change is >= tol_mark, or the problem's tol when tol_mark < 0).
+__device__ __forceinline__ void resync_report(const SigDesc &sd, int64_t t, float r32, float rt,
+                                              float z, float n, float rn, float lam,
+                                              unsigned char *__restrict__ dirty, float tol_mark,
+                                              float &zex, float &nzg, float &all, float &dz32)
 {
-    const int64_t Tz = sd.Tz;
-    // r = beta0 - (hi + lo), finished with TwoSum so that only the final
-    // float rounding remains
-    const float sm = __fsub_rn(b0, ah);
-    const float bv = __fsub_rn(sm, b0);
-    const float er = __fadd_rn(__fsub_rn(b0, __fsub_rn(sm, bv)), __fsub_rn(-ah, bv));
-    const float r32 = __fadd_rn(sm, __fsub_rn(er, al));
-    if (write_r)
-        rr[ix] = r32;
-    drift = fmaxf(drift, fabsf(rold - r32));
     // optimality in the r form (Theorem A.1): z = 0 needs |beta| = |r| <= lam;
     // otherwise |Z' - z| with Z' from Eq. pb_coord, without cancellation
     float gap;
@@ -178,13 +163,14 @@ __device__ __forceinline__ void resync_finish_v(const SigDesc &sd, int64_t ix, i
     all = fmaxf(all, fabsf(gap));
     // the phase kernel's own test on the float state it will see
     float zn, d32;
-    coord_step(write_r ? r32 : rold, z, n, rn, lam, &zn, &d32);
+    coord_step(rt, z, n, rn, lam, &zn, &d32);
     dz32 = fmaxf(dz32, fabsf(d32));
     if (dirty && sd.nseg > 0 && fabsf(d32) >= (tol_mark < 0.f ? sd.tol : tol_mark))
-        dirty[sd.seg0 + segment_of(Tz, sd.nseg, t)] = 1;
+        dirty[sd.seg0 + segment_of(sd.Tz, sd.nseg, t)] = 1;
 }
 
-// resync_finish_v with its loads
+// The refreshed r of coordinate (k, t) of problem sd from beta0 and the
+// double-float sum (ah, al) of its S Z terms, its drift |r_old - r| and report.
 __device__ __forceinline__ void resync_finish(const SigDesc &sd, int k, int64_t t,
                                               const float *__restrict__ b0p,
                                               float *__restrict__ rr,
@@ -196,9 +182,18 @@ __device__ __forceinline__ void resync_finish(const SigDesc &sd, int k, int64_t 
                                               float &dz32)
 {
     const int64_t ix = (int64_t)k * sd.ld + t;
-    const float n = norms[k];
-    resync_finish_v(sd, ix, t, b0p[ix], rr[ix], zz[ix], n, __frcp_rn(n), rr, ah, al, lam, write_r,
-                    dirty, tol_mark, drift, zex, nzg, all, dz32);
+    const float n = norms[k], b0 = b0p[ix], rold = rr[ix];
+    // r = beta0 - (hi + lo), finished with TwoSum so that only the final
+    // float rounding remains
+    const float sm = __fsub_rn(b0, ah);
+    const float bv = __fsub_rn(sm, b0);
+    const float er = __fadd_rn(__fsub_rn(b0, __fsub_rn(sm, bv)), __fsub_rn(-ah, bv));
+    const float r32 = __fadd_rn(sm, __fsub_rn(er, al));
+    if (write_r)
+        rr[ix] = r32;
+    drift = fmaxf(drift, fabsf(rold - r32));
+    resync_report(sd, t, r32, write_r ? r32 : rold, zz[ix], n, __frcp_rn(n), lam, dirty, tol_mark,
+                  zex, nzg, all, dz32);
 }
 
 // KPT = 4 NG atoms per thread: thread group g (of kResyncGroups) owns the
@@ -388,20 +383,69 @@ __global__ void __launch_bounds__(kResyncThreads, KPT <= 4 ? 3 : 1)
     }
 }
 
-// The resync with a few warps per tile (lane = column): the tiles of a long
-// signal are many and each needs little arithmetic (a few nonzeros reach a
-// 32-column tile at the optimum), so what bounds a tile is its chain of
-// dependent memory round trips; small blocks keep many tiles in flight on an
-// SM and need no barrier before the final reduction.  Block = WPT warps of
-// one tile; warp q owns the float4 atom groups [q NG, (q+1) NG) of the
-// by-lag table, and each lane loads the coefficients of NB nonzeros, and the
-// state of its NG x 4 coordinates, in one round.  The nonzeros are read from
-// the buckets in the same order as resync_kernel (bucket, then (k, column)),
-// or, when a bucket overflowed or no lists are given, gathered from Z in that
-// same order with ballots: results are identical either way.  Needs 2R+1 <=
-// 32 buckets, R = ceil((L-1)/32) (L <= 481), and K <= 64 (at most 8 warps).
+// Packed pairs of floats (two IEEE operations per instruction).  Products go
+// through fma with -0: a packed product whose only use is a packed sum is
+// otherwise contracted with it, which would break the error-free sums below.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
+{
+    unsigned long long x;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(lo), "f"(hi));
+    return x;
+}
+__device__ __forceinline__ void unpack2(unsigned long long x, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
+                                                   unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+constexpr unsigned long long kOne2 = 0x3f8000003f800000ull;
+constexpr unsigned long long kMinusOne2 = 0xbf800000bf800000ull;
+constexpr unsigned long long kMinusZero2 = 0x8000000080000000ull;
+
+// df_add_prod on two accumulators at once, negated: (hi, lo) -= a b; nb = -b.
+// (The rounded product enters TwoSum as a nb, the one form that is needed.)
+__device__ __forceinline__ void df2_sub_prod(unsigned long long &hi, unsigned long long &lo,
+                                             unsigned long long a, unsigned long long b,
+                                             unsigned long long nb)
+{
+    const unsigned long long np = fma2(a, nb, kMinusZero2);
+    const unsigned long long pe = fma2(a, b, np);                   // a b - p
+    const unsigned long long s = fma2(hi, kOne2, np);
+    const unsigned long long bv = fma2(hi, kMinusOne2, s);          // s - hi
+    const unsigned long long t1 = fma2(bv, kMinusOne2, s);          // s - bv
+    const unsigned long long t2 = fma2(t1, kMinusOne2, hi);         // hi - (s - bv)
+    const unsigned long long t3 = fma2(bv, kMinusOne2, np);         // np - bv
+    const unsigned long long e = fma2(pe, kMinusOne2, fma2(t2, kOne2, t3));
+    hi = s;
+    lo = fma2(lo, kOne2, e);
+}
+
+// The resync of a tile by a few warps (lane = column): block = WPT warps of one
+// tile, warp q owns the float4 atom groups [2 q, 2 q + 2) of the by-lag table (one
+// group where K <= 4).  The tile's nonzeros are decoded once per block into a
+// shared list of (table offset, column, z), in the order of the buckets and of
+// (k, column) inside them; each warp then walks it, two coordinates per
+// double-float instruction.  A tile whose buckets overflowed, or a call without
+// lists, gathers from Z in that same order with ballots: results are identical
+// either way.  Needs 2R+1 <= 32 buckets, R = ceil((L-1)/32) (L <= 481), and K <= 64
+// (at most 8 warps).
+//
+// What bounds it is the FP32 pipe (a packed instruction occupies it twice as long;
+// 66% busy) and issue (64%): a coordinate takes 10 to 20 products of 10 packed
+// instructions per pair, and a finish that is short where z = 0 and |r| <=
+// lambda (nearly everywhere).  P=7, K=25, L=64, T=200,000: 126 -> 82 us; the two
+// refreshes of 24 such signals (6.3 M columns) 3.20 + 1.78 -> 1.86 + 1.07 ms,
+// against the form in which every warp fetched the list with shuffles and summed
+// coordinate by coordinate.  Three or four nonzeros' coefficients in flight need
+// registers that cost a block per SM: no faster than two.
+constexpr int kEntries = 256;  // nonzeros decoded at a time
 template <int NG>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 4)
     resync_warp_kernel(const SigDesc *__restrict__ sigs, Tiles tiles, const float *__restrict__ Ct,
                        const float *__restrict__ norms, int K, int L, int write_r,
                        unsigned long long *__restrict__ red, int red_stride,
@@ -410,18 +454,18 @@ __global__ void __launch_bounds__(256, 2)
                        NzLists lists)
 {
     constexpr int KPT = 4 * NG;
-    constexpr int NB = NG == 1 ? 8 : 4;  // nonzeros whose coefficients are loaded together
+    constexpr int NB = 2;  // nonzeros whose coefficients are loaded together
     constexpr unsigned kFullMask = 0xffffffffu;
-    __shared__ float bred[5][32];
-    __shared__ int s_need;
+    __shared__ float bred[5][8];
+    __shared__ int s_off[34], s_need;
+    // table offset and lag of lane 0; z, z, -z, -z
+    __shared__ __align__(8) int2 s_ent[kEntries];
+    __shared__ __align__(16) float4 s_z[kEntries];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5, nwq = blockDim.x >> 5;
     const int64_t b = blockIdx.x;
     const int isig = tiles.sig[b];
-    const SigDesc sd = sigs[isig];
+    const SigDesc &sd = sigs[isig];
     const int64_t Tz = sd.Tz, ld = sd.ld;
-    float *__restrict__ const rr = sd.r;
-    const float *__restrict__ const zz = sd.Z;
-    const float *__restrict__ const b0p = sd.beta0;
     const int W2 = 2 * L - 1;
     const int G = (K + 3) / 4;  // float4 groups of the table
     const int g0 = wq * NG;     // this warp's first group
@@ -429,12 +473,35 @@ __global__ void __launch_bounds__(256, 2)
     const int64_t t = c0 + lane;
     const int64_t tend = tiles.end && tiles.end[b] < Tz ? tiles.end[b] : Tz;
     const bool col_ok = t < tend;
-    float drift = 0.f, zex = 0.f, nzg = 0.f, all = 0.f, dz32 = 0.f;
-    // whether the tile must be recomputed: decided once per block (the
-    // segment range of the tile takes two 64-bit divisions)
-    if (threadIdx.x == 0)
-        s_need = !(touched && rep) || tile_touched(sd, c0, touched);
+    // buckets b-R .. b+R of the same problem: lane j of the first warp holds
+    // bucket b-R+j; whether the tile must be recomputed is decided once per block
+    // (the segment range of the tile takes two 64-bit divisions)
+    const int R = (L - 1 + kResyncCols - 1) / kResyncCols;
+    if (wq == 0) {
+        int cnt = 0;
+        if (lists.count && lane <= 2 * R) {
+            const int64_t bb = b - R + lane;
+            const bool valid = bb >= 0 && bb < tiles.n && tiles.sig[bb] == isig &&
+                               tiles.start[bb] == c0 + (int64_t)(lane - R) * kResyncCols;
+            cnt = valid ? lists.count[bb] : 0;
+        }
+        const bool over = __any_sync(kFullMask, cnt > kNzCap);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFullMask, incl, o);
+            if (lane >= o)
+                incl += v;
+        }
+        s_off[lane + 1] = incl;
+        if (lane == 0) {
+            s_off[0] = 0;
+            s_off[33] = lists.count && !over;
+            s_need = !(touched && rep) || tile_touched(sd, c0, touched);
+        }
+    }
     __syncthreads();
+    float drift = 0.f, zex = 0.f, nzg = 0.f, all = 0.f, dz32 = 0.f;
     const bool need = s_need != 0;
     if (!need) {
         if (lane == 0 && wq == 0) {  // the stored report of the unchanged tile (drift 0)
@@ -444,109 +511,80 @@ __global__ void __launch_bounds__(256, 2)
             dz32 = rep[5 * b + 4];
         }
     } else {
-        // this lane's coordinates: its state first (one round trip for all)
-        float b0v[KPT], rov[KPT], zv[KPT], nv[KPT];
-        // 1 / ||D_k||^2 of the warp's KPT atoms: lane q computes atom q's
-        const int kq = 4 * (g0 + (lane % KPT) / 4) + (lane % KPT) % 4;
-        const float rn_lane = __frcp_rn(kq < K ? norms[kq] : 1.f);
+        float *__restrict__ const rr = sd.r;
+        const float *__restrict__ const zz = sd.Z;
+        const float *__restrict__ const b0p = sd.beta0;
+        unsigned long long hi[KPT / 2], lo[KPT / 2];
 #pragma unroll
-        for (int q = 0; q < KPT; q++) {
-            const int k = 4 * (g0 + q / 4) + (q % 4);
-            const bool ok = col_ok && k < K;
-            const int64_t ix = (int64_t)(ok ? k : 0) * ld + (ok ? t : 0);
-            b0v[q] = ok ? b0p[ix] : 0.f;
-            rov[q] = ok ? rr[ix] : 0.f;
-            zv[q] = ok ? zz[ix] : 0.f;
-            nv[q] = ok ? norms[k] : 1.f;
-        }
-        float acc_hi[KPT], acc_lo[KPT];
+        for (int i = 0; i < KPT / 2; i++)
+            hi[i] = lo[i] = 0ull;
+        // one nonzero (uniform over the warp): the coefficients of atom k at lag
+        // d0 + lane are float4 words base + lane + gi W2; a lane outside the
+        // window reads lag 0 and adds the exact product 0 (lanes beyond the tile's
+        // last column add what they read: nothing is written for them)
+        const ulonglong2 *const Ct2 = reinterpret_cast<const ulonglong2 *>(Ct) + g0 * W2;
+        int gstep[NG];
 #pragma unroll
-        for (int i = 0; i < KPT; i++) {
-            acc_hi[i] = 0.f;
-            acc_lo[i] = 0.f;
-        }
-        const float4 *Ct4 = reinterpret_cast<const float4 *>(Ct);
-        // NB nonzeros (k, column, z) at a time: loads first, then the sums; a
-        // nonzero out of this lane's window (z = 0 there) adds nothing
-        // (column offsets relative to the tile start c0: 32-bit)
-        auto add_batch = [&](const int (&kk)[NB], const int (&tc)[NB], const float (&z)[NB]) {
-            float4 cv[NB][NG];
-            float zz_[NB];
-#pragma unroll
-            for (int e = 0; e < NB; e++) {
-                const int d = lane - tc[e] + (L - 1);
-                const bool in = col_ok && z[e] != 0.f && d >= 0 && d < W2;
-                zz_[e] = in ? z[e] : 0.f;
-                const int base = (kk[e] * G + g0) * W2 + (in ? d : 0);
-#pragma unroll
-                for (int gi = 0; gi < NG; gi++)
-                    cv[e][gi] = in && g0 + gi < G ? __ldg(Ct4 + base + gi * W2)
-                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int e = 0; e < NB; e++)
-                if (zz_[e] != 0.f) {
-#pragma unroll
-                    for (int gi = 0; gi < NG; gi++) {
-                        df_add_prod(acc_hi[4 * gi], acc_lo[4 * gi], cv[e][gi].x, zz_[e]);
-                        df_add_prod(acc_hi[4 * gi + 1], acc_lo[4 * gi + 1], cv[e][gi].y, zz_[e]);
-                        df_add_prod(acc_hi[4 * gi + 2], acc_lo[4 * gi + 2], cv[e][gi].z, zz_[e]);
-                        df_add_prod(acc_hi[4 * gi + 3], acc_lo[4 * gi + 3], cv[e][gi].w, zz_[e]);
-                    }
+        for (int gi = 0; gi < NG; gi++)
+            gstep[gi] = (g0 + gi < G ? gi : 0) * W2;
+        // (partial: some lane of the entry's 32 is outside its window)
+        auto fetch = [&](int base, int d0, ulonglong2 zz2, ulonglong2 (&cv)[NG], ulonglong2 &z2) {
+            const ulonglong2 *p = Ct2 + (base + lane);
+            z2 = zz2;
+            if (d0 < 0 || d0 + 31 >= W2) {
+                const int d = d0 + lane;
+                if (d < 0 || d >= W2) {
+                    p = Ct2 + (base - d0);
+                    z2 = make_ulonglong2(0ull, 0ull);
                 }
-        };
-        // buckets b-R .. b+R of the same problem: lane j holds bucket b-R+j
-        const int R = (L - 1 + kResyncCols - 1) / kResyncCols;
-        int cnt = 0;
-        if (lists.count && lane <= 2 * R) {
-            const int64_t bb = b - R + lane;
-            const bool valid = bb >= 0 && bb < tiles.n && tiles.sig[bb] == isig &&
-                               tiles.start[bb] == c0 + (int64_t)(lane - R) * kResyncCols;
-            cnt = valid ? lists.count[bb] : 0;
-        }
-        const bool listed = lists.count && !__any_sync(kFullMask, cnt > kNzCap);
-        if (listed) {
-            // entries in bucket order: prefix of the counts over the lanes
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(kFullMask, incl, o);
-                if (lane >= o)
-                    incl += v;
             }
-            const int total = __shfl_sync(kFullMask, incl, 31);
-            const int excl = incl - cnt;
-            for (int e0 = 0; e0 < total; e0 += 32) {
-                // lane l fetches entry e0 + l: its bucket j is the last one with
-                // excl_j <= e (empty buckets before it are passed over)
-                const int e = e0 + lane;
-                int j = 0;
-                for (int q = 0; q <= 2 * R; q++)
-                    if (e >= __shfl_sync(kFullMask, excl, q))
-                        j = q;
-                const int xj = __shfl_sync(kFullMask, excl, j);
-                const uint2 v = e < total ? lists.ent[(b - R + j) * kNzCap + (e - xj)]
-                                          : make_uint2(0u, 0u);
-                // atom and column offset from c0 in one word: k << 16 | (offset + 1024)
-                // (offsets lie in [-32 R, 32 R + 32), 2R + 1 <= 32)
-                const int off = (j - R) * kResyncCols + (int)(v.x % kResyncCols);
-                const unsigned pk = ((v.x / kResyncCols) << 16) | (unsigned)(off + 1024);
-                const int m = total - e0 < 32 ? total - e0 : 32;
+#pragma unroll
+            for (int gi = 0; gi < NG; gi++)
+                cv[gi] = __ldg(p + gstep[gi]);
+        };
+        auto add = [&](const ulonglong2 (&cv)[NG], ulonglong2 z2) {
+#pragma unroll
+            for (int gi = 0; gi < NG; gi++) {
+                df2_sub_prod(hi[2 * gi], lo[2 * gi], cv[gi].x, z2.x, z2.y);
+                df2_sub_prod(hi[2 * gi + 1], lo[2 * gi + 1], cv[gi].y, z2.x, z2.y);
+            }
+        };
+        if (s_off[33]) {
+            const int total = s_off[2 * R + 1];
+            for (int e0 = 0; e0 < total; e0 += kEntries) {
+                const int m = total - e0 < kEntries ? total - e0 : kEntries;
+                for (int i = threadIdx.x; i < m; i += blockDim.x) {
+                    // its bucket j: the last one with s_off[j] <= e
+                    int j = 0;
+                    for (int q = 1; q <= 2 * R; q++)
+                        j = e0 + i >= s_off[q] ? q : j;
+                    const uint2 v = lists.ent[(b - R + j) * kNzCap + (e0 + i - s_off[j])];
+                    const int k = (int)(v.x / kResyncCols);
+                    const int tc = (j - R) * kResyncCols + (int)(v.x % kResyncCols);
+                    const int d0 = L - 1 - tc;  // lag of lane 0
+                    s_ent[i] = make_int2(k * G * W2 + d0, d0);
+                    const float z = __uint_as_float(v.y);
+                    s_z[i] = make_float4(z, z, -z, -z);
+                }
+                __syncthreads();
+                // NB nonzeros' coefficients in flight
                 for (int i0 = 0; i0 < m; i0 += NB) {
-                    int kk[NB];
-                    int tc[NB];
-                    float z[NB];
+                    ulonglong2 cv[NB][NG];
+                    ulonglong2 z2[NB];
 #pragma unroll
                     for (int x = 0; x < NB; x++) {
-                        const int src = i0 + x < m ? i0 + x : 0;
-                        const unsigned px = __shfl_sync(kFullMask, pk, src);
-                        const float zx = __uint_as_float(__shfl_sync(kFullMask, v.y, src));
-                        kk[x] = (int)(px >> 16);
-                        tc[x] = (int)(px & 0xffffu) - 1024;
-                        z[x] = i0 + x < m ? zx : 0.f;
+                        const int i = i0 + x < m ? i0 + x : m - 1;
+                        const int2 e = s_ent[i];
+                        fetch(e.x, e.y, *reinterpret_cast<const ulonglong2 *>(&s_z[i]), cv[x],
+                              z2[x]);
                     }
-                    add_batch(kk, tc, z);
+#pragma unroll
+                    for (int x = 0; x < NB; x++)
+                        if (i0 + x < m)
+                            add(cv[x], z2[x]);
                 }
+                if (e0 + kEntries < total)
+                    __syncthreads();  // the list is rewritten
             }
         } else {
             // from Z itself, bucket by bucket, (k, column) order by ballots;
@@ -562,34 +600,59 @@ __global__ void __launch_bounds__(256, 2)
                     const float zq = in ? zz[(int64_t)k * ld + tq] : 0.f;
                     unsigned msk = __ballot_sync(kFullMask, zq != 0.f);
                     while (msk) {
-                        int kk[NB];
-                        int tc[NB];
-                        float z[NB];
-#pragma unroll
-                        for (int x = 0; x < NB; x++) {
-                            const int src = msk ? __ffs((int)msk) - 1 : 0;
-                            const float zx = __shfl_sync(kFullMask, zq, src);
-                            kk[x] = k;
-                            tc[x] = (q - R) * kResyncCols + src;
-                            z[x] = msk ? zx : 0.f;
-                            msk &= msk - 1;
-                        }
-                        add_batch(kk, tc, z);
+                        const int src = __ffs((int)msk) - 1;
+                        const float z = __shfl_sync(kFullMask, zq, src);
+                        const int d0 = L - 1 - ((q - R) * kResyncCols + src);
+                        ulonglong2 cv[NG], z2;
+                        fetch(k * G * W2 + d0, d0,
+                              make_ulonglong2(pack2(z, z), pack2(-z, -z)), cv, z2);
+                        add(cv, z2);
+                        msk &= msk - 1;
                     }
                 }
             }
         }
+        // finish: r = beta0 - (hi + lo), finished with TwoSum so that only the
+        // final float rounding remains, and the tile's report
         const float lam = sd.lam;
+        if (col_ok) {
+            float b0v[KPT], rov[KPT], zv[KPT];
 #pragma unroll
-        for (int q = 0; q < KPT; q++) {
-            const int k = 4 * (g0 + q / 4) + (q % 4);
-            // every lane takes part in the shuffle (col_ok differs across the
-            // lanes of a signal's last tile)
-            const float rn = __shfl_sync(kFullMask, rn_lane, q);
-            if (col_ok && k < K)
-                resync_finish_v(sd, (int64_t)k * ld + t, t, b0v[q], rov[q], zv[q], nv[q], rn, rr,
-                                acc_hi[q], acc_lo[q], lam, write_r, dirty, tol_mark, drift, zex,
-                                nzg, all, dz32);
+            for (int q = 0; q < KPT; q++) {
+                const int k = 4 * g0 + q;
+                const int64_t ix = (int64_t)(k < K ? k : 0) * ld + t;
+                b0v[q] = k < K ? b0p[ix] : 0.f;
+                rov[q] = k < K ? rr[ix] : 0.f;
+                zv[q] = k < K ? zz[ix] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < KPT; q++) {
+                const int k = 4 * g0 + q;
+                if (k >= K)
+                    break;
+                float h0, h1, l0, l1;
+                unpack2(hi[q / 2], h0, h1);
+                unpack2(lo[q / 2], l0, l1);
+                // (the pair holds minus the sum)
+                const float ah = q & 1 ? -h1 : -h0, al = q & 1 ? -l1 : -l0, b0 = b0v[q];
+                const float sm = __fsub_rn(b0, ah);
+                const float bv = __fsub_rn(sm, b0);
+                const float er = __fadd_rn(__fsub_rn(b0, __fsub_rn(sm, bv)), __fsub_rn(-ah, bv));
+                const float r32 = __fadd_rn(sm, __fsub_rn(er, al));
+                if (write_r)
+                    rr[(int64_t)k * ld + t] = r32;
+                drift = fmaxf(drift, fabsf(rov[q] - r32));
+                // z = 0 and |r| <= lambda (on the state tested, too): no step, no gap
+                const float rt = write_r ? r32 : rov[q];
+                const float ex = fmaxf(fabsf(r32), fabsf(rt)) - lam;
+                if (zv[q] == 0.f && !(ex > 0.f)) {
+                    zex = fmaxf(zex, fabsf(r32) - lam);
+                    continue;
+                }
+                const float n = norms[k];
+                resync_report(sd, t, r32, rt, zv[q], n, __frcp_rn(n), lam, dirty, tol_mark, zex,
+                              nzg, all, dz32);
+            }
         }
     }
     for (int off = 16; off > 0; off >>= 1) {
@@ -616,7 +679,8 @@ __global__ void __launch_bounds__(256, 2)
                 rep[5 * b + q] = v[q];
         unsigned long long *rd = red + (int64_t)isig * red_stride;
         for (int q = 0; q < 5; q++)
-            atomicMax(&rd[q], (unsigned long long)__double_as_longlong((double)v[q]));
+            if (v[q] > 0.f)
+                atomicMax(&rd[q], (unsigned long long)__double_as_longlong((double)v[q]));
     }
 }
 
