@@ -21,14 +21,15 @@
 // N = 1 is the paper's cut along one axis (bands only); more column blocks
 // give more co-active tiles, which one GPU needs (a 512 x 512 image with
 // 8 x 8 atoms has 18 co-active bands but 324 co-active tiles of 14 x 14).
-// One thread block per active tile: it keeps, per position (i, j) of its
-// tile, the best coordinate over k as a 64-bit key (|Delta Z| bits, ~flat
-// index and the sign of Delta Z; ties to the lowest (k Hz + i) Wz + j) in
-// shared memory, with r and Z of the tile staged there too when they fit, and
-// repeats block argmax (a shared atomicMax per warp, one barrier) -> update
-// -> re-evaluation of the window's positions, writing the window positions
-// outside its tile (idle neighbours) with atomicAdd and each new Z value to
-// global memory when it is applied.
+// One thread block per active tile; the automatic tiles of at most 32 atoms run in
+// csc2d_tile.cuh, the others (more atoms, large windows, bands) in tile_kernel: it
+// keeps, per position (i, j) of its tile, the best coordinate over k as a 64-bit
+// key (|Delta Z| bits, ~flat index and the sign of Delta Z; ties to the lowest
+// (k Hz + i) Wz + j) in shared memory, with r and Z of the tile staged there too
+// when they fit, and repeats block argmax (a shared atomicMax per warp, one
+// barrier) -> update -> re-evaluation of the window's positions, writing the
+// window positions outside its tile (idle neighbours) with atomicAdd and each new
+// Z value to global memory when it is applied.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -164,16 +165,46 @@ struct TileParams {
     Dims d;
     int Mr, Mc, KQ, u;
     int max_pos;             // positions of the largest tile (shared-memory layout)
+    int max_ext;             // the same with h-1 rows and w-1 columns on every side
     float lam, tol;
 };
 
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long v)
 {
     unsigned hi = (unsigned)(v >> 32);
     const unsigned hmax = __reduce_max_sync(0xffffffffu, hi);
     unsigned lo = hi == hmax ? (unsigned)v : 0u;
     const unsigned lmax = __reduce_max_sync(0xffffffffu, lo);
     return ((unsigned long long)hmax << 32) | lmax;
+}
+
+// End of a tile's visit (one thread): its flag, the tiles that its updates' windows
+// (around the rows [imin, imax] and columns [jmin, jmax]) reached, the counts.
+__device__ __forceinline__ void tile_done(const TileParams &tp, int tile, int m, int n, int nupd,
+                                          bool capped, double dsum, int64_t imin, int64_t imax,
+                                          int64_t jmin, int64_t jmax)
+{
+    const Dims &d = tp.d;
+    tp.dirty[tile] = capped ? 1 : 0;
+    if (nupd == 0)
+        return;
+    const int64_t rlo = imin - (d.h - 1), rhi = imax + (d.h - 1);
+    const int64_t clo = jmin - (d.w - 1), chi = jmax + (d.w - 1);
+    int m0 = m, m1 = m, n0 = n, n1 = n;
+    while (m0 > 0 && tp.row_s[m0] > rlo)
+        m0--;
+    while (m1 + 1 < tp.Mr && tp.row_s[m1 + 1] <= rhi)
+        m1++;
+    while (n0 > 0 && tp.col_s[n0] > clo)
+        n0--;
+    while (n1 + 1 < tp.Mc && tp.col_s[n1 + 1] <= chi)
+        n1++;
+    for (int mm = m0; mm <= m1; mm++)
+        for (int nn = n0; nn <= n1; nn++)
+            if (mm != m || nn != n)
+                tp.dirty[mm * tp.Mc + nn] = 1;
+    atomicAdd(reinterpret_cast<unsigned long long *>(tp.upd), (unsigned long long)nupd);
+    atomicAdd(tp.dec, dsum);
 }
 
 // Shared-memory layout of a tile block (bytes, 16-aligned pieces): per
@@ -328,7 +359,7 @@ __global__ void __launch_bounds__(kB2, 3) tile_kernel(TileParams tp)
                 my = kk > my ? kk : my;
             });
         });
-        const unsigned long long wm = warp_max_u64(my);
+        const unsigned long long wm = warp_max_key(my);
         if (lane == 0 && wm != 0ull)
             atomicMax(&s_best[it & 3], wm);
         if (tid == 0)
@@ -422,29 +453,15 @@ __global__ void __launch_bounds__(kB2, 3) tile_kernel(TileParams tp)
         double dsum = 0.0;
         for (int q = 0; q < kB2 / 32; q++)
             dsum += s_dec[q];
-        tp.dirty[tile] = capped ? 1 : 0;
-        if (nupd > 0) {
-            // tiles the windows reached need a visit again
-            const int64_t rlo = imin - (d.h - 1), rhi = imax + (d.h - 1);
-            const int64_t clo = jmin - (d.w - 1), chi = jmax + (d.w - 1);
-            int m0 = m, m1 = m, n0 = n, n1 = n;
-            while (m0 > 0 && tp.row_s[m0] > rlo)
-                m0--;
-            while (m1 + 1 < tp.Mr && tp.row_s[m1 + 1] <= rhi)
-                m1++;
-            while (n0 > 0 && tp.col_s[n0] > clo)
-                n0--;
-            while (n1 + 1 < tp.Mc && tp.col_s[n1 + 1] <= chi)
-                n1++;
-            for (int mm = m0; mm <= m1; mm++)
-                for (int nn = n0; nn <= n1; nn++)
-                    if (mm != m || nn != n)
-                        tp.dirty[mm * tp.Mc + nn] = 1;
-            atomicAdd(reinterpret_cast<unsigned long long *>(tp.upd), (unsigned long long)nupd);
-            atomicAdd(tp.dec, dsum);
-        }
+        tile_done(tp, tile, m, n, nupd, capped, dsum, imin, imax, jmin, jmax);
     }
 }
+
+}  // namespace
+
+#include "csc2d_tile.cuh"
+
+namespace {
 
 // ---------------------------------------------------------------- exact checks
 
@@ -939,14 +956,25 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     };
     if (max_pos >= ((int64_t)1 << 31) / 64 || bits(hmax - 1) + bits(wmax - 1) > 25)
         return csc_record_error(CSC_EINVAL, "csc2d_solve: tiles too large");
+    // thread-private positions (csc2d_tile.cuh) where one group of threads holds a
+    // position's atoms, the window has a thread per position, and the tile with
+    // its halo fits shared memory, a 32-bit mask of a thread's positions and the
+    // key's index word; else (many atoms, large windows, bands) tile_kernel
+    const int A = (2 * h - 1) * (2 * w - 1), nq = (K + 3) / 4;
+    const int64_t max_ext = (hmax + 2 * h - 2) * (wmax + 2 * w - 2);
+    const size_t reg_smem = tile_reg_smem(nq, max_ext, max_pos);
+    const int64_t nslots = ((hmax + 4 * h - 4) / (2 * h - 1)) * ((wmax + 4 * w - 4) / (2 * w - 1));
+    const bool reg = K <= 32 && A <= 512 && reg_smem <= (size_t)kMaxSmem - 4096 && nslots <= 32 &&
+                     bits(hmax - 1) + bits(wmax - 1) <= 24;
     // a tile's r and Z are staged in shared memory when they fit
     const bool stage = TileLayout(K, (int)max_pos, true).total <= (size_t)kMaxSmem;
-    const size_t smem = TileLayout(K, (int)max_pos, stage).total;
+    const size_t smem = reg ? reg_smem : TileLayout(K, (int)max_pos, stage).total;
     if (smem > (size_t)kMaxSmem)
         return csc_record_error(CSC_EINVAL,
                                 "csc2d_solve: a tile of %lld x %lld positions needs %zu bytes of "
                                 "shared memory (more bands or column blocks)",
                                 (long long)hmax, (long long)wmax, smem);
+    const int block = reg ? ((A + 31) & ~31) + 32 : kB2;
     // the exact checks gather the nonzeros of (2h-1) rows x K atoms one column
     // chunk at a time: one column must fit the list; the objective's
     // channels are spread over 8 thread groups, at most 8 passes each
@@ -959,7 +987,6 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     Dev2 g;
     const int KQ = (K + 3) / 4;
     const int64_t nz = (int64_t)K * d.Hz * d.Wz;
-    const int A = (2 * h - 1) * (2 * w - 1);
     const int64_t ntile_o = H * ((W + kTile2 - 1) / kTile2);
     const int64_t ntc = (d.Wz + kTile2 - 1) / kTile2, nbk = d.Hz * ntc;
     {
@@ -1042,7 +1069,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
         C2_CUDA(cudaGetLastError());
         launches += 2;
     }
-    auto tile_fn = stage ? tile_kernel<true> : tile_kernel<false>;
+    auto tile_fn = reg ? tile_reg_fn(K, block) : stage ? tile_kernel<true> : tile_kernel<false>;
     C2_CUDA(cudaFuncSetAttribute(tile_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
     TileParams tp;
@@ -1060,6 +1087,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     tp.Mc = Nb;
     tp.KQ = KQ;
     tp.max_pos = (int)max_pos;
+    tp.max_ext = (int)max_ext;
     tp.u = updates_per_visit > 0 ? updates_per_visit : kAutoVisit2d;
     tp.lam = (float)lambda;
     const int max_resyncs = 3;
@@ -1089,7 +1117,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                     if (cnt == 0)
                         continue;
                     tp.list = g.list + off[p];
-                    tile_fn<<<cnt, kB2, smem, s>>>(tp);
+                    tile_fn<<<cnt, block, smem, s>>>(tp);
                     C2_CUDA(cudaGetLastError());
                     launches++;
                 }

@@ -45,200 +45,21 @@
 #pragma once
 
 #include "csc_internal.cuh"
+#include "phase_rank.cuh"
 #include "phase_reg.cuh"
 
 namespace csc {
 
 namespace {
 
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRegWarps = 16;  // column warps of a block at most (and one active warp)
 constexpr int kRegAtoms = 32 * kRegWarps;  // padded atoms: at most 16 groups of 8 float4
-constexpr int kActive = 128;   // listed coordinates of a visit at most
 
-// x, hidden from the optimiser: keeps multiples of a stride from being hoisted
-// out of the update loop into registers.
-__device__ __forceinline__ int64_t opaque(int64_t x)
-{
-    asm volatile("" : "+l"(x));
-    return x;
-}
-__device__ __forceinline__ int opaque(int x)
-{
-    asm volatile("" : "+r"(x));
-    return x;
-}
-
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned hi, unsigned lo)
-{
-    const unsigned hmax = __reduce_max_sync(kFull, hi);
-    const unsigned lmax = __reduce_max_sync(kFull, hi == hmax ? lo : 0u);
-    return ((unsigned long long)hmax << 32) | lmax;
-}
-
-// Index word of a key, complemented so that the largest key is the lowest
-// (atom, column): k << 17 | slot << 12 | class << 2 | listed << 1 | sign of dZ.
-__device__ __forceinline__ unsigned key_index(unsigned k, unsigned pos, unsigned listed,
-                                              unsigned neg)
-{
-    return ~((k << 17) | pos | (listed << 1) | neg);
-}
+// Index word of a key (key_index, atoms from bit 17 on): the column's bits.
+constexpr int kKeyShift = 17;
 __device__ __forceinline__ unsigned key_pos(unsigned slot, unsigned c)
 {
     return (slot << 12) | (c << 2);
-}
-
-// Packed pairs of floats (one 64-bit register pair, two operations at once).
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
-{
-    unsigned long long x;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(lo), "f"(hi));
-    return x;
-}
-__device__ __forceinline__ void unpack2(unsigned long long x, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
-{
-    // (scalar: the packed sum of a packed product would be contracted)
-    float a0, a1, b0, b1;
-    unpack2(a, a0, a1);
-    unpack2(b, b0, b1);
-    return pack2(__fadd_rn(a0, b0), __fadd_rn(a1, b1));
-}
-
-// A column's r (atom rows src + i ld, n of them) copied to shared memory in the
-// background (cp.async, completed by halo_wait in the same thread).
-template <int N>
-__device__ __forceinline__ void halo_load(unsigned long long *dst, const float *src, int64_t ld,
-                                          int n)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    const int64_t step = opaque(ld);
-#pragma unroll
-    for (int i = 0; i < N; i++, src += step)
-        if (i < n)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * i),
-                         "l"(__cvta_generic_to_global(src))
-                         : "memory");
-}
-template <int N>
-__device__ __forceinline__ void halo_store(const unsigned long long *src, float *dst, int64_t ld,
-                                           int n)
-{
-    const int64_t step = opaque(ld);
-#pragma unroll
-    for (int i = 0; i < N; i += 2) {
-        float lo, hi;
-        unpack2(src[i / 2], lo, hi);
-        if (i < n)
-            *dst = lo;
-        dst += step;
-        if (i + 1 < n)
-            *dst = hi;
-        dst += step;
-    }
-}
-__device__ __forceinline__ void halo_wait()
-{
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
-// v = (|r| - lam) / n of the two atoms of a pair (rn: 1 / n)
-__device__ __forceinline__ void excess2(unsigned long long r, unsigned long long rn, float lam,
-                                        float &v0, float &v1)
-{
-    float a, b;
-    unpack2(r, a, b);
-    unpack2(mul2(pack2(fabsf(a) - lam, fabsf(b) - lam), rn), v0, v1);
-}
-
-// The best of one column's atoms with z == 0 from v[i] = (|r_i| - lambda) / n_i
-// (NaN for atoms on the active list): its key, 0 when nothing moves.  r: the
-// staged column.  coord_step's float32 resolution floor can reject the best
-// only when its excess over lambda is a few ulps; then all are tested.
-template <int N>
-__device__ __forceinline__ void rank_column(const float (&v)[N], const float *r, const float *rn,
-                                            float lam, unsigned kbase, unsigned pos,
-                                            unsigned &khi, unsigned &klo)
-{
-    constexpr float kFloor = 4.76837158203125e-07f;  // 2^-21
-    // (four chains, so that their latencies overlap)
-    float m[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < N; i += 2) {
-        float &x = m[(i >> 1) & 3];
-        x = fmaxf(x, fmaxf(v[i], v[i + 1]));
-    }
-    float vm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
-    khi = 0u;
-    klo = 0u;
-    if (vm > 0.f) {
-        // the first atom that attains it
-        int b[2] = {N, N};
-#pragma unroll
-        for (int i = N / 2 - 1; i >= 0; i--) {
-            if (v[i] == vm)
-                b[0] = i;
-            if (v[i + N / 2] == vm)
-                b[1] = i + N / 2;
-        }
-        int bi = min(b[0], b[1]);
-        float rs = r[bi];
-        if (vm < fabsf(rs) * kFloor * rn[bi]) {
-            vm = 0.f;
-#pragma unroll 1
-            for (int i = 0; i < N; i++) {
-                const float y = r[i], x = (fabsf(y) - lam) * rn[i];
-                if (x > vm && !(x < fabsf(y) * kFloor * rn[i])) {
-                    vm = x;
-                    bi = i;
-                    rs = y;
-                }
-            }
-        }
-        if (vm > 0.f) {
-            khi = __float_as_uint(vm);
-            klo = key_index(kbase + bi, pos, 0u, __float_as_uint(rs) >> 31);
-        }
-    }
-}
-
-// Adds the coordinates of a column whose Z is nonzero but not listed (bits of
-// zm) to its key (khi, klo); r: the staged column, zcol + i ld: Z of atom kbase + i.
-__device__ __forceinline__ void rank_unlisted(unsigned zm, const float *r, const float *zcol,
-                                              int64_t ld, const float *nrm, const float *rn,
-                                              float lam,
-                                              unsigned kbase, unsigned pos, unsigned &khi,
-                                              unsigned &klo)
-{
-#pragma unroll 1
-    for (; zm; zm &= zm - 1) {
-        const int i = __ffs((int)zm) - 1;
-        float zn, d;
-        coord_step(r[i], zcol[(int64_t)i * ld], nrm[i], rn[i], lam, &zn, &d);
-        const unsigned h = __float_as_uint(fabsf(d));
-        const unsigned l = key_index(kbase + i, pos, 0u, d < 0.f ? 1u : 0u);
-        if (fabsf(d) > 0.f && (h > khi || (h == khi && l > klo))) {
-            khi = h;
-            klo = l;
-        }
-    }
 }
 
 // One launch of a phase.  drain == 0: block b visits segment phase_list[b];
@@ -375,8 +196,12 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 const int64_t step = opaque(ld);
                 const unsigned pos = key_pos((unsigned)s, (unsigned)c);
                 unsigned zb = 0, zl = 0;
+                float v[N];  // (r and Z in one round trip)
                 {
-                    const float *zp = zbase + jj;
+                    const float *rp = rbase + jj, *zp = zbase + jj;
+#pragma unroll
+                    for (int i = 0; i < N; i++, rp += step)
+                        v[i] = (int)kbase + i < K ? *rp : 0.f;
 #pragma unroll
                     for (int i = 0; i < N; i++, zp += step)
                         zb |= ((int)kbase + i < K && *zp != 0.f ? 1u : 0u) << i;
@@ -392,13 +217,6 @@ __global__ void __launch_bounds__(MAXT, MINB)
                     }
                 }
                 zb &= ~zl;
-                float v[N];
-                {
-                    const float *rp = rbase + jj;
-#pragma unroll
-                    for (int i = 0; i < N; i++, rp += step)
-                        v[i] = (int)kbase + i < K ? *rp : 0.f;
-                }
 #pragma unroll
                 for (int i = 0; i < N; i++)
                     if (zl >> i & 1u)
@@ -420,9 +238,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
                             v[i] = -1.f;
                 }
                 const float *const rc = reinterpret_cast<const float *>(col);
-                rank_column<N>(v, rc, rn, lam, kbase, pos, khi, klo);
+                rank_column<N>(v, rc, rn, lam, zb, kbase, kKeyShift, pos, khi, klo);
                 if (zb)
-                    rank_unlisted(zb, rc, zbase + jj, ld, nrm, rn, lam, kbase, pos, khi, klo);
+                    rank_unlisted(zb, rc, zbase + jj, ld, nrm, rn, lam, kbase, kKeyShift, pos, khi,
+                                  klo);
                 skey[jj] = ((unsigned long long)khi << 32) | klo;
                 slst[jj] = zl;
                 sunl[jj] = zb;
@@ -622,10 +441,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
                                 if (zb >> i & 1u)
                                     v[i] = -1.f;
                         }
-                        rank_column<N>(v, rc, rn, lam, kbase, pos, khi, klo);
+                        rank_column<N>(v, rc, rn, lam, zb, kbase, kKeyShift, pos, khi, klo);
                         if (zb)
-                            rank_unlisted(zb, rc, zbase + jj, ld, nrm, rn, lam, kbase, pos, khi,
-                                          klo);
+                            rank_unlisted(zb, rc, zbase + jj, ld, nrm, rn, lam, kbase, kKeyShift, pos,
+                                          khi, klo);
                         skey[jj] = ((unsigned long long)khi << 32) | klo;
                     } else {
                         // an idle neighbour's column: its r, product and sum
