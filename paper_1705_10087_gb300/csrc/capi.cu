@@ -720,9 +720,8 @@ int csc_init_batch(csc_handle_t h, const float *X, const int64_t *T, int n, cons
         CSC_CUDA(cudaEventCreate(&h->ev_i0));
         CSC_CUDA(cudaEventCreate(&h->ev_i1));
     }
-    // a cold start (Z = 0) has r = beta0: the kernel writes both, and the
-    // tensor-core kernel also zeroes Z and, for a batch, takes the per-signal
-    // maxima (the kernel's overall maximum also covers the columns between
+    // a cold start (Z = 0) has r = beta0: the kernel writes both and zeroes Z;
+    // the tensor-core kernel also, for a batch, takes the per-signal maxima (the kernel's overall maximum also covers the columns between
     // signals, which belong to no problem)
     Dtx0Extras ex;
     if (!Z0)
@@ -756,8 +755,6 @@ int csc_init_batch(csc_handle_t h, const float *X, const int64_t *T, int n, cons
         CSC_CUDA(cudaMemsetAsync(h->sc->red, 0, sizeof(h->sc->red), s));
         CSC_CUDA(launch_resync(h->d_sig, h->resync_tiles(), h->Ct, h->norms, h->K, h->L, 1,
                                h->sc->red, 0, nullptr, 0.f, nullptr, nullptr, h->nz_lists(), s));
-    } else if (!ex.done) {
-        CSC_CUDA(cudaMemsetAsync(h->Z, 0, sizeof(float) * nz, s));
     }
     // read back without waiting (finish_init completes it): the stream goes
     // on to the solve while beta0 is computed

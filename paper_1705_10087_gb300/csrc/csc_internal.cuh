@@ -270,7 +270,7 @@ cudaError_t launch_expand_tiles(const int64_t *off, int n, int width, int64_t co
 
 cudaError_t launch_dtx(const float *D, const float *X, int K, int P, int L, int64_t T,
                        float *beta0, float *r_out, unsigned int *absmax_bits, double *x2sum,
-                       cudaStream_t s);
+                       cudaStream_t s, float *z_out = nullptr);
 
 // Reduction / output tiles of a batch: tile b covers columns (or samples)
 // [start[b], start[b] + width) of problem sig[b], clipped to the problem and,
@@ -300,7 +300,7 @@ inline bool dtx_tc_preferred(int K, int P, int L)
 // pass: z_out != NULL zeroes Z [K][Tz] (a cold start); lmax != NULL gathers the
 // maximum |beta0| of each of the nsig problems of a batch (float bits, zeroed
 // by the caller), problem i owning the columns [a[i], a[i+1] - L + 1).  done
-// is set when the kernel that ran did both (the FP32 kernel does neither).
+// is set when the kernel that ran did the maxima (the FP32 kernel only zeroes Z).
 struct Dtx0Extras {
     float *z_out = nullptr;
     const int64_t *a = nullptr;  // [nsig + 1] first sample of each problem (device)

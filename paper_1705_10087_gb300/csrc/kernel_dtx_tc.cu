@@ -717,7 +717,8 @@ cudaError_t launch_dtx_any(const float *D, const float *X, int K, int P, int L, 
             return e;
         cudaGetLastError();
     }
-    return launch_dtx(D, X, K, P, L, T, beta0, r_out, absmax_bits, x2sum, s);
+    return launch_dtx(D, X, K, P, L, T, beta0, r_out, absmax_bits, x2sum, s,
+                      ex ? ex->z_out : nullptr);
 }
 
 }  // namespace csc

@@ -901,14 +901,25 @@ __global__ void __launch_bounds__(kTile)
         atomicMax(&out[i], __float_as_uint(m));
 }
 
-__global__ void beta_from_r_kernel(const float *__restrict__ r, const float *__restrict__ Z,
-                                   const float *__restrict__ norms, int K, int64_t Tz,
-                                   float *__restrict__ out)
+// (grid row k: atom k's row; a block takes 1024 columns, four per thread in
+// flight)
+__global__ void __launch_bounds__(256)
+    beta_from_r_kernel(const float *__restrict__ r, const float *__restrict__ Z,
+                       const float *__restrict__ norms, int64_t Tz, float *__restrict__ out)
 {
-    const int64_t n = (int64_t)K * Tz;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = fmaf(norms[i / Tz], Z[i], r[i]);
+    const int64_t o = blockIdx.y * Tz, i0 = blockIdx.x * (int64_t)1024 + threadIdx.x;
+    const float n = norms[blockIdx.y];
+    float z[4], x[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const int64_t i = i0 + 256 * q;
+        z[q] = i < Tz ? Z[o + i] : 0.f;
+        x[q] = i < Tz ? r[o + i] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+        if (i0 + 256 * q < Tz)
+            out[o + i0 + 256 * q] = fmaf(n, z[q], x[q]);
 }
 
 template <int KPT>
@@ -983,10 +994,8 @@ cudaError_t launch_resync(const SigDesc *sig, Tiles tiles, const float *Ct, cons
 cudaError_t launch_beta_from_r(const float *r, const float *Z, const float *norms, int K,
                                int64_t Tz, float *out, cudaStream_t s)
 {
-    const int64_t n = (int64_t)K * Tz;
-    const int64_t grid = (n + 255) / 256;
-    beta_from_r_kernel<<<(unsigned)(grid < 152 * 64 ? grid : 152 * 64), 256, 0, s>>>(r, Z, norms,
-                                                                                   K, Tz, out);
+    beta_from_r_kernel<<<dim3((unsigned)((Tz + 1023) / 1024), (unsigned)K), 256, 0, s>>>(
+        r, Z, norms, Tz, out);
     return cudaGetLastError();
 }
 

@@ -12,16 +12,23 @@ namespace csc {
 namespace {
 
 // DtD[k0][k][s] = sum_p sum_tau D[k][p][tau] * D[k0][p][tau + s - (L-1)]
-// = S_{k,k0}[s-(L-1)] of Eq. beta_up (Sec. 2.1).  One block per pair (k0, k),
+// = S_{k,k0}[s-(L-1)] of Eq. beta_up (Sec. 2.1).  One block per pair (k0, k <= k0),
 // one thread per lag; with STAGE the two atoms are first copied to shared
-// memory (every thread of the block reads all of both).
+// memory (every thread of the block reads all of both).  The pair (k, k0) is the
+// same at the mirrored lag, term by term, and is written along.
 template <bool STAGE>
 __global__ void dtd_kernel(const float *__restrict__ D, int K, int P, int L,
                            float *__restrict__ C, float *__restrict__ norms)
 {
     extern __shared__ float dsm[];  // STAGE: [2][P][L], atom k then atom k0
     const int W2 = 2 * L - 1;
-    const int k0 = blockIdx.x / K, k = blockIdx.x % K;
+    // pair number b = k0 (k0 + 1) / 2 + k
+    int k0 = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while (k0 * (k0 + 1) / 2 > (int)blockIdx.x)
+        k0--;
+    while ((k0 + 1) * (k0 + 2) / 2 <= (int)blockIdx.x)
+        k0++;
+    const int k = blockIdx.x - k0 * (k0 + 1) / 2;
     const int PL = P * L;
     const float *da = D + (long long)k * PL, *db = D + (long long)k0 * PL;
     if (STAGE) {
@@ -53,6 +60,7 @@ __global__ void dtd_kernel(const float *__restrict__ D, int K, int P, int L,
         }
         const float v = acc.value();
         C[((long long)k0 * K + k) * W2 + s] = v;
+        C[((long long)k * K + k0) * W2 + (W2 - 1 - s)] = v;
         if (k == k0 && lag == 0)
             norms[k] = v;
     }
@@ -67,14 +75,19 @@ constexpr int kDtxAtoms = 8;                        // atoms per block
 // plus max |beta0| (lambda_max) and sum X^2 (2 E(0)).  Block: 1024 consecutive
 // t and 8 atoms; a thread owns 4 consecutive t, so each 8-lag step reads 12
 // samples of X (3 vector loads) and the 8 atoms' 8 lags (broadcast vector
-// loads) for 256 FMAs.  Lags are padded to a multiple of 8 with zeros.
-__global__ void __launch_bounds__(kDtxThreads) dtx_kernel(const float *__restrict__ D,
-                                                         const float *__restrict__ X, int K,
-                                                         int P, int L, long long T,
-                                                         float *__restrict__ beta0,
-                                                         float *__restrict__ r_out,
-                                                         unsigned int *__restrict__ absmax_bits,
-                                                         double *__restrict__ x2sum)
+// loads) for 256 FMAs.  Lags are padded to a multiple of 8 with zeros.  What
+// bounds it is issue (75% busy; 256 FMAs and 128 compensation sums of the 403
+// instructions of a step).  Samples and atoms come in the background, all in flight
+// together: K=64, P=7, L=64, T=300,007 608 -> 560 us (two atoms per packed
+// instruction: 587 us, the FP32 pipe takes a packed one at less than twice the rate).
+__global__ void __launch_bounds__(kDtxThreads, 2) dtx_kernel(const float *__restrict__ D,
+                                                            const float *__restrict__ X, int K,
+                                                            int P, int L, long long T,
+                                                            float *__restrict__ beta0,
+                                                            float *__restrict__ r_out,
+                                                            float *__restrict__ z_out,
+                                                            unsigned int *__restrict__ absmax_bits,
+                                                            double *__restrict__ x2sum)
 {
     extern __shared__ __align__(16) float sm[];
     const int L8 = (L + 7) & ~7;
@@ -86,21 +99,36 @@ __global__ void __launch_bounds__(kDtxThreads) dtx_kernel(const float *__restric
     const int k0 = blockIdx.y * kDtxAtoms;
     const int nk = min(kDtxAtoms, K - k0);
 
-    double x2 = 0.0;
-    const bool last = t0 + kDtxTile >= Tz;  // the last block also owns samples [Tz, T)
-    for (int i = threadIdx.x; i < P * xw; i += blockDim.x) {
-        const int p = i / xw, j = i % xw;
-        const long long t = t0 + j;
-        const float v = t < T ? X[(long long)p * T + t] : 0.f;
-        xs[i] = v;
-        if (blockIdx.y == 0 && (j < kDtxTile || last))
-            x2 += (double)v * (double)v;
+    // the samples and the atoms on their way together (zeros beyond the ends)
+    auto fetch = [](float *dst, const float *src, bool ok) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(dst)),
+                     "l"(__cvta_generic_to_global(src)), "r"(ok ? 4 : 0)
+                     : "memory");
+    };
+    for (int p = 0; p < P; p++)
+        for (int j = threadIdx.x; j < xw; j += kDtxThreads) {
+            const bool ok = t0 + j < T;
+            fetch(xs + p * xw + j, X + (ok ? (long long)p * T + t0 + j : 0), ok);
+        }
+    // a warp stages one atom's row of lags at a time
+    for (int i = threadIdx.x >> 5; i < kDtxAtoms * P; i += kDtxThreads / 32) {
+        const int kk = i / P, p = i - kk * P;
+        for (int tau = threadIdx.x & 31; tau < L8; tau += 32) {
+            const bool ok = kk < nk && tau < L;
+            fetch(ds + i * L8 + tau,
+                  D + (ok ? ((long long)(k0 + kk) * P + p) * L + tau : 0), ok);
+        }
     }
-    for (int i = threadIdx.x; i < kDtxAtoms * P * L8; i += blockDim.x) {
-        const int kk = i / (P * L8), r = i % (P * L8), p = r / L8, tau = r % L8;
-        ds[i] = (kk < nk && tau < L) ? D[((long long)(k0 + kk) * P + p) * L + tau] : 0.f;
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    double x2 = 0.0;
+    if (blockIdx.y == 0) {
+        const bool last = t0 + kDtxTile >= Tz;  // the last block also owns samples [Tz, T)
+        for (int p = 0; p < P; p++)
+            for (int j = threadIdx.x; j < (last ? xw : kDtxTile); j += kDtxThreads)
+                x2 += (double)xs[p * xw + j] * (double)xs[p * xw + j];
+    }
 
     const int j4 = threadIdx.x * kDtxT;
     KahanF acc[kDtxAtoms][kDtxT];
@@ -142,9 +170,12 @@ __global__ void __launch_bounds__(kDtxThreads) dtx_kernel(const float *__restric
             for (int kk = 0; kk < kDtxAtoms; kk++) {
                 if (kk < nk) {
                     const float v = acc[kk][q].value();
-                    beta0[(long long)(k0 + kk) * Tz + t] = v;
+                    const long long o = (long long)(k0 + kk) * Tz + t;
+                    beta0[o] = v;
                     if (r_out)
-                        r_out[(long long)(k0 + kk) * Tz + t] = v;
+                        r_out[o] = v;
+                    if (z_out)
+                        z_out[o] = 0.f;
                     amax = fmaxf(amax, fabsf(v));
                 }
             }
@@ -191,9 +222,9 @@ cudaError_t launch_dtd(const float *D, int K, int P, int L, float *C, float *nor
     const int block = W2 <= 128 ? 128 : (W2 <= 256 ? 256 : 512);
     const size_t smem = 2 * sizeof(float) * (size_t)P * L;
     if (smem <= 48 * 1024)
-        dtd_kernel<true><<<(unsigned)(K * K), block, smem, s>>>(D, K, P, L, C, norms);
+        dtd_kernel<true><<<(unsigned)(K * (K + 1) / 2), block, smem, s>>>(D, K, P, L, C, norms);
     else
-        dtd_kernel<false><<<(unsigned)(K * K), block, 0, s>>>(D, K, P, L, C, norms);
+        dtd_kernel<false><<<(unsigned)(K * (K + 1) / 2), block, 0, s>>>(D, K, P, L, C, norms);
     return cudaGetLastError();
 }
 
@@ -234,7 +265,7 @@ cudaError_t launch_expand_tiles(const int64_t *off, int n, int width, int64_t co
 
 cudaError_t launch_dtx(const float *D, const float *X, int K, int P, int L, int64_t T,
                        float *beta0, float *r_out, unsigned int *absmax_bits, double *x2sum,
-                       cudaStream_t s)
+                       cudaStream_t s, float *z_out)
 {
     const int L8 = (L + 7) & ~7;
     const size_t smem =
@@ -247,8 +278,8 @@ cudaError_t launch_dtx(const float *D, const float *X, int K, int P, int L, int6
         return e;
     const int64_t Tz = T - L + 1;
     dim3 grid((unsigned)((Tz + kDtxTile - 1) / kDtxTile), (unsigned)((K + kDtxAtoms - 1) / kDtxAtoms));
-    dtx_kernel<<<grid, kDtxThreads, smem, s>>>(D, X, K, P, L, T, beta0, r_out, absmax_bits,
-                                               x2sum);
+    dtx_kernel<<<grid, kDtxThreads, smem, s>>>(D, X, K, P, L, T, beta0, r_out, z_out,
+                                               absmax_bits, x2sum);
     return cudaGetLastError();
 }
 

@@ -261,15 +261,15 @@ int admit(csc_server_t s, Group &g, double t)
         q.r = reinterpret_cast<float *>(b);
         b += align_up(sizeof(float) * g.K * q.Tz);
         q.Z = reinterpret_cast<float *>(b);
-        const size_t nz = sizeof(float) * g.K * q.Tz;
         SRV_CUDA(cudaMemcpyAsync(q.X, q.Xh.data(), sizeof(float) * g.P * q.T,
                                  cudaMemcpyHostToDevice, g.st));
         SRV_CUDA(cudaMemsetAsync(q.hdr, 0, sizeof(ReqHeader), g.st));
-        // Z = 0: r = beta0, written by the same kernel
+        // Z = 0: r = beta0, both written by the same kernel
+        Dtx0Extras ex;
+        ex.z_out = q.Z;
         SRV_CUDA(launch_dtx_any(g.D, q.X, g.K, g.P, g.L, q.T, 0, q.beta0, q.r,
-                                &q.hdr->lmax_bits, &q.hdr->x2, &q.hdr->tc_err, g.st));
+                                &q.hdr->lmax_bits, &q.hdr->x2, &q.hdr->tc_err, g.st, &ex));
         s->launches += 1;
-        SRV_CUDA(cudaMemsetAsync(q.Z, 0, nz, g.st));
         q.state = CSC_REQ_ACTIVE;
         q.t_admit = t;
         g.queue.pop_front();
