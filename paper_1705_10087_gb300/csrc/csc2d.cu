@@ -38,6 +38,7 @@
 #include "csc2d.h"
 #include "csc_internal.cuh"
 #include "host_util.cuh"
+#include "packed.cuh"
 
 using namespace csc;
 
@@ -111,43 +112,82 @@ __global__ void dtd2d_kernel(const float *__restrict__ D, Dims d, int KQ, float 
     }
 }
 
-// beta0 (and r = beta0 for Z = 0) in double-float sums rounded once (the
-// FP64 pipe of GB300 is narrow); max |beta0| and sum X^2 (E(0) = sum X^2 / 2).
-__global__ void dtx2d_kernel(const float *__restrict__ D, const float *__restrict__ X, Dims d,
-                             float *__restrict__ beta0, float *__restrict__ r,
-                             unsigned *__restrict__ absmax, double *__restrict__ x2)
+// beta0, r = beta0 and Z = 0 in double-float sums rounded once (the FP64 pipe of
+// GB300 is narrow); max |beta0| and sum X^2 (E(0) = sum X^2 / 2).  A thread takes a
+// position and the 8 atoms of its grid row, two per instruction, so a sample is
+// loaded once for 8 products and the atoms of a channel come from shared memory.
+// Bound by the FP32 pipe.  512 x 512 image, 8 atoms of 8 x 8: 91 us with a thread
+// per coordinate, 47 us.
+constexpr int kAtoms2 = 8;
+__global__ void __launch_bounds__(256)
+    dtx2d_kernel(const float *__restrict__ D, const float *__restrict__ X, Dims d,
+                 float *__restrict__ beta0, float *__restrict__ r, float *__restrict__ Z,
+                 unsigned *__restrict__ absmax, double *__restrict__ x2)
 {
-    const int64_t n = (int64_t)d.K * d.Hz * d.Wz;
-    float amax = 0.f;
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n;
-         o += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = o % d.Wz, i = (o / d.Wz) % d.Hz;
-        const int k = (int)(o / (d.Wz * d.Hz));
-        float hi = 0.f, lo = 0.f;
-        for (int p = 0; p < d.P; p++)
-            for (int u = 0; u < d.h; u++) {
-                const float *xr = X + ((int64_t)p * d.H + i + u) * d.W + j;
-                const float *dr = D + (((int64_t)k * d.P + p) * d.h + u) * d.w;
-                for (int v = 0; v < d.w; v++)
-                    df_add_prod(hi, lo, __ldg(dr + v), __ldg(xr + v));
+    extern __shared__ __align__(16) float ds[];  // [h w][kAtoms2] of one channel
+    const int k0 = blockIdx.y * kAtoms2, hw = d.h * d.w;
+    const int64_t HWz = d.Hz * d.Wz;
+    const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool ok = o < HWz;
+    const int64_t i = ok ? o / d.Wz : 0, j = ok ? o - i * d.Wz : 0;
+    unsigned long long hi[kAtoms2 / 2], lo[kAtoms2 / 2];  // minus the sums
+#pragma unroll
+    for (int a = 0; a < kAtoms2 / 2; a++)
+        hi[a] = lo[a] = 0ull;
+    for (int p = 0; p < d.P; p++) {
+        if (p)
+            __syncthreads();
+        for (int e = threadIdx.x; e < hw * kAtoms2; e += blockDim.x) {
+            const int a = e & (kAtoms2 - 1), uv = e / kAtoms2;
+            ds[e] = k0 + a < d.K ? D[((int64_t)(k0 + a) * d.P + p) * hw + uv] : 0.f;
+        }
+        __syncthreads();
+        if (!ok)
+            continue;
+        const float *xr = X + ((int64_t)p * d.H + i) * d.W + j;
+        const ulonglong2 *dv = reinterpret_cast<const ulonglong2 *>(ds);
+        for (int u = 0; u < d.h; u++, xr += d.W)
+#pragma unroll 4
+            for (int v = 0; v < d.w; v++, dv += 2) {
+                const float x = __ldg(xr + v);
+                const unsigned long long x2v = pack2(x, x), nx = pack2(-x, -x);
+                const ulonglong2 a = dv[0], b = dv[1];
+                df2_sub_prod(hi[0], lo[0], a.x, x2v, nx);
+                df2_sub_prod(hi[1], lo[1], a.y, x2v, nx);
+                df2_sub_prod(hi[2], lo[2], b.x, x2v, nx);
+                df2_sub_prod(hi[3], lo[3], b.y, x2v, nx);
             }
-        const float b = __fadd_rn(hi, lo);
-        beta0[o] = b;
-        r[o] = b;
-        amax = fmaxf(amax, fabsf(b));
     }
+    float amax = 0.f;
+    if (ok)
+#pragma unroll
+        for (int a = 0; a < kAtoms2; a++) {
+            if (k0 + a >= d.K)
+                break;
+            float h0, h1, l0, l1;
+            unpack2(hi[a / 2], h0, h1);
+            unpack2(lo[a / 2], l0, l1);
+            const float b = a & 1 ? __fadd_rn(-h1, -l1) : __fadd_rn(-h0, -l0);
+            const int64_t at = (k0 + a) * HWz + o;
+            beta0[at] = b;
+            r[at] = b;
+            Z[at] = 0.f;
+            amax = fmaxf(amax, fabsf(b));
+        }
     double s = 0.0;
-    const int64_t nx = (int64_t)d.P * d.H * d.W;
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < nx;
-         o += (int64_t)gridDim.x * blockDim.x)
-        s += (double)X[o] * (double)X[o];
+    if (blockIdx.y == 0) {
+        const int64_t nx = (int64_t)d.P * d.H * d.W;
+        for (int64_t e = o; e < nx; e += (int64_t)gridDim.x * blockDim.x)
+            s += (double)X[e] * (double)X[e];
+    }
     for (int off = 16; off > 0; off >>= 1) {
         amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
         s += __shfl_xor_sync(0xffffffffu, s, off);
     }
     if ((threadIdx.x & 31) == 0) {
         atomicMax(absmax, __float_as_uint(amax));
-        atomicAdd(x2, s);
+        if (blockIdx.y == 0)
+            atomicAdd(x2, s);
     }
 }
 
@@ -613,51 +653,71 @@ __device__ int gather2(const Buckets2 &bk, int64_t r0, int64_t r1, int64_t c0, i
     return total;
 }
 
-// r = beta0 - sum C Z (FP64 sums) on one row and kTile2 columns per block
-// (threads: 32 columns x 8 atom groups), and the optimality report as in 1-D:
-// red[0] drift, red[3] max |Delta Z| (no floor), red[4] the coordinate step on
-// the refreshed state (with the float32 floor); write_r = 0 leaves r alone.
+// Rows of the output that a block of 8 warps takes when a row's positions need
+// `warps` of them (kTile2 columns each); fewer where more rows would take the
+// region's buckets beyond kGather2 (w - 1 columns more on either side) or the
+// elements of one column beyond the list.
+inline int rows_per_block(int warps, int K, int region_rows, int w)
+{
+    const int nt = (kTile2 + 2 * w - 2) / kTile2 + 2;
+    int rb = warps >= 8 ? 1 : 8 / warps;
+    while (rb > 1 && ((int64_t)K * (region_rows + rb - 1) > kList2 ||
+                      (region_rows + rb - 1) * nt > kGather2))
+        rb--;
+    return rb;
+}
+
+// r = beta0 - sum C Z (double-float sums) on rb rows and kTile2 columns per block
+// (a warp: 32 columns of one row and one or, for K > 32, two float4 groups of
+// atoms), and the optimality report as in 1-D: red[0] drift, red[3] max |Delta Z|
+// (no floor), red[4] the coordinate step on the refreshed state (with the float32
+// floor); write_r = 0 leaves r alone.  A listed nonzero costs a lane one 128-bit
+// coefficient load and two packed double-float sums per group; with a thread per
+// (column, 8 atom groups) of one row every atom's thread walked the list on its
+// own (512 x 512 image, 8 atoms of 8 x 8: 240 -> 64 us).
 __global__ void __launch_bounds__(256)
     resync2d_kernel(const float *__restrict__ beta0, float *__restrict__ r,
                     const float *__restrict__ Z, const float *__restrict__ Ct,
-                    const float *__restrict__ norms, Dims d, int KQ, float lam, int write_r,
-                    Buckets2 bk, unsigned long long *__restrict__ red)
+                    const float *__restrict__ norms, Dims d, int KQ, int rb, float lam,
+                    int write_r, Buckets2 bk, unsigned long long *__restrict__ red)
 {
     __shared__ NZ2 list[kList2];
     __shared__ int wc[8];
     __shared__ float bred[3][8];
     __shared__ int s_cnt[kGather2], s_off[kGather2 + 1], s_flag;
-    const int tid = threadIdx.x, col = tid & 31, grp = tid >> 5;
+    const int tid = threadIdx.x, col = tid & 31, warp = tid >> 5;
     const int64_t ntc = (d.Wz + kTile2 - 1) / kTile2;
-    const int64_t i = blockIdx.x / ntc, j0 = (blockIdx.x % ntc) * kTile2, j = j0 + col;
+    const int64_t i0 = blockIdx.x / ntc * rb, j0 = (blockIdx.x % ntc) * kTile2, j = j0 + col;
+    const int wpr = KQ < 8 ? KQ : 8;  // warps per row
+    const int64_t i = i0 + warp / wpr;
+    const int q0 = warp % wpr;
+    const bool on = warp / wpr < rb && i < d.Hz && j < d.Wz;
     const int H2 = 2 * d.h - 1, W2 = 2 * d.w - 1, A = H2 * W2;
-    const int64_t r0 = max((int64_t)0, i - (d.h - 1)), r1 = min(d.Hz, i + d.h);
+    const int64_t r0 = max((int64_t)0, i0 - (d.h - 1)), r1 = min(d.Hz, i0 + rb - 1 + d.h);
     const int64_t c0 = max((int64_t)0, j0 - (d.w - 1)), c1 = min(d.Wz, j0 + kTile2 + d.w - 1);
-    constexpr int kPer = (kMaxK2 + 7) / 8;
-    float acc_hi[kPer], acc_lo[kPer];  // double-float sums of C z
+    unsigned long long hi[2][2], lo[2][2];  // minus the double-float sums of C z
 #pragma unroll
-    for (int q = 0; q < kPer; q++) {
-        acc_hi[q] = 0.f;
-        acc_lo[q] = 0.f;
-    }
+    for (int q = 0; q < 2; q++)
+        hi[q][0] = hi[q][1] = lo[q][0] = lo[q][1] = 0ull;
     // sum C z over the listed nonzeros whose window holds (i, j)
     auto accumulate = [&](int n) {
-        if (j >= d.Wz)
+        if (!on)
             return;
-        for (int q = 0; q < n; q++) {
-            const NZ2 e = list[q];
-            const int a = (int)(i - e.i) + (d.h - 1), b = (int)(j - e.j) + (d.w - 1);
+        for (int e = 0; e < n; e++) {
+            const NZ2 v = list[e];
+            const int a = (int)(i - v.i) + (d.h - 1), b = (int)(j - v.j) + (d.w - 1);
             if (a < 0 || a >= H2 || b < 0 || b >= W2)
                 continue;
-            const int lag = a * W2 + b;
+            const unsigned long long z2 = pack2(v.z, v.z), nz2 = pack2(-v.z, -v.z);
 #pragma unroll
-            for (int t = 0; t < kPer; t++) {
-                const int k = grp + 8 * t;
-                if (k < d.K)
-                    df_add_prod(acc_hi[t], acc_lo[t],
-                                __ldg(Ct + ((((int64_t)e.k * KQ + (k >> 2)) * A + lag) << 2) +
-                                      (k & 3)),
-                                e.z);
+            for (int q = 0; q < 2; q++) {
+                const int g = q0 + 8 * q;
+                if (g < KQ) {
+                    const ulonglong2 c = __ldg(reinterpret_cast<const ulonglong2 *>(Ct) +
+                                               ((int64_t)v.k * KQ + g) * A + a * W2 + b);
+                    df2_sub_prod(hi[q][0], lo[q][0], c.x, z2, nz2);
+                    df2_sub_prod(hi[q][1], lo[q][1], c.y, z2, nz2);
+                }
             }
         }
     };
@@ -675,23 +735,29 @@ __global__ void __launch_bounds__(256)
         }
     }
     float drift = 0.f, all = 0.f, dz32 = 0.f;
-    if (j < d.Wz) {
+    if (on) {
 #pragma unroll
-        for (int t = 0; t < kPer; t++) {
-            const int k = grp + 8 * t;
+        for (int t = 0; t < 8; t++) {
+            const int k = 4 * (q0 + 8 * (t / 4)) + t % 4;
             if (k >= d.K)
                 continue;
             const int64_t o = ((int64_t)k * d.Hz + i) * d.Wz + j;
+            float h0, h1, l0, l1;
+            unpack2(hi[t / 4][t % 4 / 2], h0, h1);
+            unpack2(lo[t / 4][t % 4 / 2], l0, l1);
             // r = beta0 - (hi + lo), finished with TwoSum: one final rounding
             float rn = beta0[o], rl = 0.f;
-            df_add(rn, rl, -acc_hi[t]);
-            df_add(rn, rl, -acc_lo[t]);
+            df_add(rn, rl, t & 1 ? h1 : h0);
+            df_add(rn, rl, t & 1 ? l1 : l0);
             rn = __fadd_rn(rn, rl);
             const float rold = r[o];
             if (write_r)
                 r[o] = rn;
             drift = fmaxf(drift, fabsf(rold - rn));
-            const float z = Z[o], nk = norms[k], rnk = __frcp_rn(nk);
+            const float z = Z[o];
+            if (z == 0.f && fabsf(rn) <= lam)
+                continue;  // no step, no gap
+            const float nk = norms[k], rnk = __frcp_rn(nk);
             float gap;
             if (z == 0.f) {
                 gap = soft_f(rn, lam) * rnk;
@@ -712,9 +778,9 @@ __global__ void __launch_bounds__(256)
         dz32 = fmaxf(dz32, __shfl_xor_sync(0xffffffffu, dz32, off));
     }
     if (col == 0) {
-        bred[0][grp] = drift;
-        bred[1][grp] = all;
-        bred[2][grp] = dz32;
+        bred[0][warp] = drift;
+        bred[1][warp] = all;
+        bred[2][warp] = dz32;
     }
     __syncthreads();
     if (tid == 0) {
@@ -728,27 +794,34 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Residual of one image row and kTile2 columns (all channels) per block, FP64:
-// partial[2b] = sum over its pixels of R^2, partial[2b+1] = sum |Z| over the
-// block's own activation positions (rows < Hz, columns < Wz).
+// Residual of rb image rows and kTile2 columns (all channels) per block (a warp: 32
+// columns of one row, channels p, p + 8, ...), double-float per thread, FP64 per
+// warp: partial[2b] = sum over its pixels of R^2, partial[2b+1] = sum |Z| over the
+// block's own activation positions (rows < Hz, columns < Wz).  With one row per
+// block seven of eight warps of a gray image had no channel (512 x 512: 147 -> 32
+// us).
 __global__ void __launch_bounds__(256)
     objective2d_kernel(const float *__restrict__ D, const float *__restrict__ X,
-                       const float *__restrict__ Z, Dims d, Buckets2 bk,
+                       const float *__restrict__ Z, Dims d, int rb, Buckets2 bk,
                        double *__restrict__ partial)
 {
     __shared__ NZ2 list[kList2];
     __shared__ int wc[8];
     __shared__ double bsum[2][8];
     __shared__ int s_cnt[kGather2], s_off[kGather2 + 1], s_flag;
-    const int tid = threadIdx.x, col = tid & 31, grp = tid >> 5;
+    const int tid = threadIdx.x, col = tid & 31, warp = tid >> 5;
     const int64_t ntc = (d.W + kTile2 - 1) / kTile2;
-    const int64_t y = blockIdx.x / ntc, x0 = (blockIdx.x % ntc) * kTile2, x = x0 + col;
+    const int64_t y0 = blockIdx.x / ntc * rb, x0 = (blockIdx.x % ntc) * kTile2, x = x0 + col;
+    const int wpr = d.P < 8 ? d.P : 8;  // warps per row
+    const int64_t y = y0 + warp / wpr;
+    const int grp = warp % wpr;
+    const bool on = warp / wpr < rb && y < d.H && x < d.W;
     // activations reaching pixel (y, x): rows [y-h+1, y], columns [x-w+1, x]
-    const int64_t r0 = max((int64_t)0, y - (d.h - 1)), r1 = min(d.Hz, y + 1);
+    const int64_t r0 = max((int64_t)0, y0 - (d.h - 1)), r1 = min(d.Hz, y0 + rb);
     const int64_t c0 = max((int64_t)0, x0 - (d.w - 1)), c1 = min(d.Wz, x0 + kTile2);
     // double-float per thread (the FP64 pipe is narrow); FP64 per warp
     float sq_h = 0.f, sq_l = 0.f, l1_h = 0.f, l1_l = 0.f;
-    constexpr int kPm = 8;  // channels per thread group pass (P up to 64)
+    constexpr int kPm = 8;  // channels per thread (P up to 64)
     float acc_hi[kPm], acc_lo[kPm];
 #pragma unroll
     for (int t = 0; t < kPm; t++) {
@@ -757,11 +830,11 @@ __global__ void __launch_bounds__(256)
     }
     // sum D z over the listed nonzeros whose atom covers (y, x)
     auto accumulate = [&](int n) {
-        if (x >= d.W)
+        if (!on)
             return;
         for (int q = 0; q < n; q++) {
             const NZ2 e = list[q];
-            const int64_t u = y - e.i, v = x - e.j;
+            const int u = (int)(y - e.i), v = (int)(x - e.j);
             if (u < 0 || u >= d.h || v < 0 || v >= d.w)
                 continue;
 #pragma unroll
@@ -787,7 +860,7 @@ __global__ void __launch_bounds__(256)
             }
         }
     }
-    if (x < d.W)
+    if (on) {
 #pragma unroll
         for (int t = 0; t < kPm; t++) {
             const int p = grp + 8 * t;
@@ -795,10 +868,11 @@ __global__ void __launch_bounds__(256)
                 df_add_sq_residual(sq_h, sq_l, X[((int64_t)p * d.H + y) * d.W + x], acc_hi[t],
                                    acc_lo[t]);
         }
-    // |Z| of this block's own positions (row y, columns [x0, x0+32)), once
-    if (grp == 0 && y < d.Hz && x < d.Wz)
-        for (int k = 0; k < d.K; k++)
-            df_add(l1_h, l1_l, fabsf(Z[((int64_t)k * d.Hz + y) * d.Wz + x]));
+        // |Z| of this block's own positions, once
+        if (grp == 0 && y < d.Hz && x < d.Wz)
+            for (int k = 0; k < d.K; k++)
+                df_add(l1_h, l1_l, fabsf(Z[((int64_t)k * d.Hz + y) * d.Wz + x]));
+    }
     for (int off = 16; off > 0; off >>= 1) {
         const float a = __shfl_xor_sync(0xffffffffu, sq_h, off);
         const float b = __shfl_xor_sync(0xffffffffu, sq_l, off);
@@ -808,8 +882,8 @@ __global__ void __launch_bounds__(256)
         df_add_df(l1_h, l1_l, c, e);
     }
     if (col == 0) {
-        bsum[0][grp] = (double)sq_h + (double)sq_l;
-        bsum[1][grp] = (double)l1_h + (double)l1_l;
+        bsum[0][warp] = (double)sq_h + (double)sq_l;
+        bsum[1][warp] = (double)l1_h + (double)l1_l;
     }
     __syncthreads();
     if (tid == 0) {
@@ -987,7 +1061,10 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     Dev2 g;
     const int KQ = (K + 3) / 4;
     const int64_t nz = (int64_t)K * d.Hz * d.Wz;
-    const int64_t ntile_o = H * ((W + kTile2 - 1) / kTile2);
+    // rows per block of the exact refresh and of the objective
+    const int rb_r = rows_per_block(KQ, K, 2 * h - 1, w),
+              rb_o = rows_per_block(P, K, h, w);
+    const int64_t ntile_o = (H + rb_o - 1) / rb_o * ((W + kTile2 - 1) / kTile2);
     const int64_t ntc = (d.Wz + kTile2 - 1) / kTile2, nbk = d.Hz * ntc;
     {
         // one allocation, pieces on 256-byte boundaries
@@ -1053,7 +1130,6 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                             s));
     C2_CUDA(cudaMemsetAsync(g.amax, 0, sizeof(unsigned), s));
     C2_CUDA(cudaMemsetAsync(g.x2, 0, sizeof(double), s));
-    C2_CUDA(cudaMemsetAsync(g.Z, 0, sizeof(float) * nz, s));
     C2_CUDA(cudaMemsetAsync(g.dirty, 1, ntiles, s));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     C2_CUDA(cudaEventCreate(&e0));
@@ -1064,8 +1140,10 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
         dtd2d_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(g.D, d, KQ,
                                                                                        g.Ct, g.norms);
         C2_CUDA(cudaGetLastError());
-        dtx2d_kernel<<<(unsigned)std::min<int64_t>((nz + 255) / 256, 152 * 16), 256, 0, s>>>(
-            g.D, g.X, d, g.beta0, g.r, g.amax, g.x2);
+        dtx2d_kernel<<<dim3((unsigned)((d.Hz * d.Wz + 255) / 256),
+                            (unsigned)((K + kAtoms2 - 1) / kAtoms2)),
+                       256, sizeof(float) * kAtoms2 * h * w, s>>>(g.D, g.X, d, g.beta0, g.r, g.Z,
+                                                                  g.amax, g.x2);
         C2_CUDA(cudaGetLastError());
         launches += 2;
     }
@@ -1095,7 +1173,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     int64_t updates = 0, sweeps = 0;
     int resyncs = 0;
     bool converged = false;
-    const unsigned rgrid = (unsigned)(d.Hz * ntc);
+    const unsigned rgrid = (unsigned)((d.Hz + rb_r - 1) / rb_r * ntc);
     const Buckets2 bk2{g.bcount, g.bent, ntc};
     double dz32 = 0.0, all = 0.0;
     for (;;) {
@@ -1140,7 +1218,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                                                                          g.bent);
         C2_CUDA(cudaGetLastError());
         resync2d_kernel<<<rgrid, 256, 0, s>>>(g.beta0, g.r, g.Z, g.Ct, g.norms, d, KQ,
-                                              (float)lambda, 1, bk2, g.red);
+                                              rb_r, (float)lambda, 1, bk2, g.red);
         C2_CUDA(cudaGetLastError());
         launches += 2;
         unsigned long long red[8];
@@ -1161,7 +1239,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     }
     C2_CUDA(cudaEventRecord(e1, s));
     const unsigned ogrid = (unsigned)ntile_o;
-    objective2d_kernel<<<ogrid, 256, 0, s>>>(g.D, g.X, g.Z, d, bk2, g.partial);  // Z as refreshed
+    objective2d_kernel<<<ogrid, 256, 0, s>>>(g.D, g.X, g.Z, d, rb_o, bk2, g.partial);  // Z as refreshed
     C2_CUDA(cudaGetLastError());
     sum_partials_kernel<<<1, 256, 0, s>>>(g.partial, ntile_o, lambda, g.E);
     C2_CUDA(cudaGetLastError());

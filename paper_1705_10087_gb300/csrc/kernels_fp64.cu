@@ -8,6 +8,7 @@
 // and every thread accumulates its outputs over that list in double-float
 // (pairs of floats with error-free transformations), combined in FP64.
 #include "csc_internal.cuh"
+#include "packed.cuh"
 
 namespace csc {
 
@@ -381,48 +382,6 @@ __global__ void __launch_bounds__(kResyncThreads, KPT <= 4 ? 3 : 1)
         for (int q = 0; q < 5; q++)
             atomicMax(&rd[q], (unsigned long long)__double_as_longlong((double)v[q]));
     }
-}
-
-// Packed pairs of floats (two IEEE operations per instruction).  Products go
-// through fma with -0: a packed product whose only use is a packed sum is
-// otherwise contracted with it, which would break the error-free sums below.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
-{
-    unsigned long long x;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(lo), "f"(hi));
-    return x;
-}
-__device__ __forceinline__ void unpack2(unsigned long long x, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-constexpr unsigned long long kOne2 = 0x3f8000003f800000ull;
-constexpr unsigned long long kMinusOne2 = 0xbf800000bf800000ull;
-constexpr unsigned long long kMinusZero2 = 0x8000000080000000ull;
-
-// df_add_prod on two accumulators at once, negated: (hi, lo) -= a b; nb = -b.
-// (The rounded product enters TwoSum as a nb, the one form that is needed.)
-__device__ __forceinline__ void df2_sub_prod(unsigned long long &hi, unsigned long long &lo,
-                                             unsigned long long a, unsigned long long b,
-                                             unsigned long long nb)
-{
-    const unsigned long long np = fma2(a, nb, kMinusZero2);
-    const unsigned long long pe = fma2(a, b, np);                   // a b - p
-    const unsigned long long s = fma2(hi, kOne2, np);
-    const unsigned long long bv = fma2(hi, kMinusOne2, s);          // s - hi
-    const unsigned long long t1 = fma2(bv, kMinusOne2, s);          // s - bv
-    const unsigned long long t2 = fma2(t1, kMinusOne2, hi);         // hi - (s - bv)
-    const unsigned long long t3 = fma2(bv, kMinusOne2, np);         // np - bv
-    const unsigned long long e = fma2(pe, kMinusOne2, fma2(t2, kOne2, t3));
-    hi = s;
-    lo = fma2(lo, kOne2, e);
 }
 
 // The resync of a tile by a few warps (lane = column): block = WPT warps of one

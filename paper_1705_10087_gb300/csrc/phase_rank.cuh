@@ -4,6 +4,7 @@
 #pragma once
 
 #include "csc_internal.cuh"
+#include "packed.cuh"
 
 namespace csc {
 
@@ -37,40 +38,6 @@ __device__ __forceinline__ unsigned key_index(unsigned k, int shift, unsigned po
                                               unsigned neg)
 {
     return ~((k << shift) | pos | (listed << 1) | neg);
-}
-
-// Packed pairs of floats (one 64-bit register pair, two operations at once).
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
-{
-    unsigned long long x;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(lo), "f"(hi));
-    return x;
-}
-__device__ __forceinline__ void unpack2(unsigned long long x, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
-{
-    // (scalar: the packed sum of a packed product would be contracted)
-    float a0, a1, b0, b1;
-    unpack2(a, a0, a1);
-    unpack2(b, b0, b1);
-    return pack2(__fadd_rn(a0, b0), __fadd_rn(a1, b1));
 }
 
 // A column's r (atom rows src + i ld, n of them) copied to shared memory in the
