@@ -62,8 +62,9 @@ int csc2d_plan(int64_t Hz, int h, int M, int *M_out, int *phases, int64_t *start
  * from Z = 0 to |Delta Z| < tol, with up to 3 exact re-synchronisations of
  * beta (FP64 sums from beta0 = D~ * X) that decide convergence, then the FP64
  * objective.  The state is float32 (the same numerics as csc_solve: the
- * float32 resolution floor applies).  The call allocates its device memory
- * on the current device and frees it before returning.
+ * float32 resolution floor applies).  The call takes its device memory on the
+ * current device; up to 64 MiB of it in all stays with the library for later
+ * calls (given back when an allocation of the library fails).
  *   D [K][P][h][w], X [P][H][W]: host or device, caller-owned
  *   1 <= K <= 64, P <= 64, K (2h-1) <= 2048, (2h-1)(2w-1) <= 4096; a tile's
  *   positions times 20 bytes must fit shared memory (about 226 KB; its r and

@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "csc2d.h"
@@ -936,9 +937,102 @@ int auto_bands(int64_t Hz, int h)
     return (int)std::max<int64_t>(1, std::min<int64_t>(Hz / bh, 1 << 20));
 }
 
-// Device buffers of one csc2d_solve call, carved from one allocation.
+// Workspaces kept between calls: a finished call leaves its device block (and 512
+// bytes of pinned memory for read-backs) for the next one, because cudaMalloc,
+// cudaFree and the synchronisation they imply took 0.3 to 0.4 ms of a call.  At most
+// kKeep2 bytes are kept in all (the oldest go first; larger blocks are freed at
+// once), and all of them are given back when an allocation of this library fails
+// (csc_trim_workspaces).  A block belongs to one call at a time and is only put
+// back after its stream was waited for, so threads and streams never share one.
+constexpr size_t kKeep2 = (size_t)64 << 20;
+constexpr size_t kPin2 = 512;
+struct Block2 {
+    void *dev = nullptr;
+    size_t cap = 0;
+    int device = 0;
+    unsigned long long *pin = nullptr;
+};
+struct Kept2 {
+    std::mutex mutex;
+    std::vector<Block2> blocks;  // oldest first
+};
+Kept2 &kept2()
+{
+    static Kept2 *k = new Kept2;  // (never destroyed: no order at exit to mind)
+    return *k;
+}
+
+void free_block2(const Block2 &b)
+{
+    csc::DeviceGuard guard(b.device);
+    cudaFree(b.dev);
+    cudaFreeHost(b.pin);
+    cudaGetLastError();
+}
+
+cudaError_t take_block2(int device, size_t bytes, Block2 *out)
+{
+    {
+        Kept2 &k = kept2();
+        std::lock_guard<std::mutex> lock(k.mutex);
+        for (size_t i = 0; i < k.blocks.size(); i++) {
+            const Block2 b = k.blocks[i];
+            // (no more than four times what is asked for)
+            if (b.device != device || b.cap < bytes || b.cap / 4 > bytes + (1 << 20))
+                continue;
+            k.blocks.erase(k.blocks.begin() + i);
+            // memory that a device reset has taken away is no block
+            cudaPointerAttributes at;
+            if (cudaPointerGetAttributes(&at, b.dev) != cudaSuccess ||
+                at.type != cudaMemoryTypeDevice || at.device != device) {
+                cudaGetLastError();
+                break;
+            }
+            *out = b;
+            return cudaSuccess;
+        }
+    }
+    Block2 b;
+    b.device = device;
+    b.cap = bytes;
+    cudaError_t e = csc::device_alloc(&b.dev, bytes);
+    if (e != cudaSuccess)
+        return e;
+    e = cudaHostAlloc(reinterpret_cast<void **>(&b.pin), kPin2, cudaHostAllocDefault);
+    if (e != cudaSuccess) {
+        cudaFree(b.dev);
+        return e;
+    }
+    *out = b;
+    return cudaSuccess;
+}
+
+void keep_block2(const Block2 &b)
+{
+    std::vector<Block2> drop;
+    if (b.cap > kKeep2) {
+        drop.push_back(b);
+    } else {
+        Kept2 &k = kept2();
+        std::lock_guard<std::mutex> lock(k.mutex);
+        k.blocks.push_back(b);
+        size_t total = 0;
+        for (const Block2 &x : k.blocks)
+            total += x.cap;
+        while (total > kKeep2) {
+            total -= k.blocks.front().cap;
+            drop.push_back(k.blocks.front());
+            k.blocks.erase(k.blocks.begin());
+        }
+    }
+    for (const Block2 &x : drop)
+        free_block2(x);
+}
+
+// Device buffers of one csc2d_solve call, carved from one block.
 struct Dev2 {
-    void *base = nullptr;
+    Block2 block;
+    bool finished = false;  // the call's stream was waited for at its end
     float *D = nullptr, *X = nullptr, *Ct = nullptr, *norms = nullptr, *beta0 = nullptr,
           *r = nullptr, *Z = nullptr;
     int64_t *band_s = nullptr, *col_s = nullptr;
@@ -950,10 +1044,30 @@ struct Dev2 {
     unsigned long long *red = nullptr;
     int *bcount = nullptr;  // nonzero buckets of Z (bucket2d_kernel)
     NZ2 *bent = nullptr;
-    ~Dev2() { cudaFree(base); }
+    ~Dev2()
+    {
+        if (!block.dev)
+            return;
+        if (finished)
+            keep_block2(block);
+        else
+            free_block2(block);  // (waits for what is still in flight)
+    }
 };
 
 }  // namespace
+
+void csc_trim_workspaces()
+{
+    std::vector<Block2> drop;
+    {
+        Kept2 &k = kept2();
+        std::lock_guard<std::mutex> lock(k.mutex);
+        drop.swap(k.blocks);
+    }
+    for (const Block2 &x : drop)
+        free_block2(x);
+}
 
 extern "C" {
 
@@ -1066,26 +1180,31 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
               rb_o = rows_per_block(P, K, h, w);
     const int64_t ntile_o = (H + rb_o - 1) / rb_o * ((W + kTile2 - 1) / kTile2);
     const int64_t ntc = (d.Wz + kTile2 - 1) / kTile2, nbk = d.Hz * ntc;
+    size_t oband = 0, ocol = 0, olist = 0, oupd = 0, ocounters = 0;
     {
-        // one allocation, pieces on 256-byte boundaries
+        // one block, pieces on 256-byte boundaries
         size_t arena = 0;
         auto piece = [&arena](size_t bytes) {
             const size_t o = arena;
             arena += (bytes + 255) & ~(size_t)255;
             return o;
         };
+        // (the tables uploaded together come first, then the counters cleared together)
+        oband = piece(sizeof(int64_t) * (Mb + 1));
+        ocol = piece(sizeof(int64_t) * (Nb + 1));
+        olist = piece(sizeof(int) * ntiles);
+        oupd = piece(sizeof(long long) * kSweepBatch);
+        const size_t odec = piece(sizeof(double)), ox2 = piece(sizeof(double)),
+                     oamax = piece(sizeof(unsigned)), ored = piece(sizeof(unsigned long long) * 8);
+        ocounters = arena - oupd;
         const size_t oD = piece(sizeof(float) * K * P * h * w), oX = piece(sizeof(float) * P * H * W),
                      oCt = piece(sizeof(float) * K * KQ * 4 * A), onorms = piece(sizeof(float) * K),
                      obeta0 = piece(sizeof(float) * nz), o_r = piece(sizeof(float) * nz),
-                     oZ = piece(sizeof(float) * nz), oband = piece(sizeof(int64_t) * (Mb + 1)),
-                     ocol = piece(sizeof(int64_t) * (Nb + 1)), olist = piece(sizeof(int) * ntiles),
-                     odirty = piece((size_t)ntiles), oupd = piece(sizeof(long long) * kSweepBatch),
-                     odec = piece(sizeof(double)), ox2 = piece(sizeof(double)),
-                     oamax = piece(sizeof(unsigned)), ored = piece(sizeof(unsigned long long) * 8),
+                     oZ = piece(sizeof(float) * nz), odirty = piece((size_t)ntiles),
                      oE = piece(sizeof(double)), opart = piece(sizeof(double) * 2 * ntile_o),
                      obc = piece(sizeof(int) * nbk), obe = piece(sizeof(NZ2) * kBucket2 * nbk);
-        C2_CUDA(cudaMalloc(&g.base, arena));
-        char *b = static_cast<char *>(g.base);
+        C2_CUDA(take_block2(dev, arena, &g.block));
+        char *b = static_cast<char *>(g.block.dev);
         g.D = reinterpret_cast<float *>(b + oD);
         g.X = reinterpret_cast<float *>(b + oX);
         g.Ct = reinterpret_cast<float *>(b + oCt);
@@ -1112,24 +1231,23 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     C2_CUDA(copy_in(g.X, X, sizeof(float) * P * H * W, s));
     // phase lists: phase pr cc + pc holds the tiles (m, n) with m == pr (mod
     // cr) and n == pc (mod cc), consecutive in the device list
-    std::vector<int> list;
+    std::vector<char> tables(oupd);  // band starts, column starts, lists: one upload
+    std::memcpy(tables.data() + oband, bs.data(), sizeof(int64_t) * (Mb + 1));
+    std::memcpy(tables.data() + ocol, cs.data(), sizeof(int64_t) * (Nb + 1));
+    int *const list = reinterpret_cast<int *>(tables.data() + olist);
     std::vector<int> off(c + 1, 0);
+    int listed = 0;
     for (int pr = 0; pr < cr; pr++)
         for (int pc = 0; pc < cc; pc++) {
-            off[pr * cc + pc] = (int)list.size();
+            off[pr * cc + pc] = listed;
             for (int m = pr; m < Mb; m += cr)
                 for (int q = pc; q < Nb; q += cc)
-                    list.push_back(m * Nb + q);
+                    list[listed++] = m * Nb + q;
         }
-    off[c] = (int)list.size();
-    C2_CUDA(cudaMemcpyAsync(g.band_s, bs.data(), sizeof(int64_t) * (Mb + 1),
-                            cudaMemcpyHostToDevice, s));
-    C2_CUDA(cudaMemcpyAsync(g.col_s, cs.data(), sizeof(int64_t) * (Nb + 1),
-                            cudaMemcpyHostToDevice, s));
-    C2_CUDA(cudaMemcpyAsync(g.list, list.data(), sizeof(int) * ntiles, cudaMemcpyHostToDevice,
-                            s));
-    C2_CUDA(cudaMemsetAsync(g.amax, 0, sizeof(unsigned), s));
-    C2_CUDA(cudaMemsetAsync(g.x2, 0, sizeof(double), s));
+    off[c] = listed;
+    C2_CUDA(cudaMemcpyAsync(g.band_s, tables.data(), oupd, cudaMemcpyHostToDevice, s));
+    // sweep counters, objective decrease, sum X^2, max |beta0|, report
+    C2_CUDA(cudaMemsetAsync(g.upd, 0, ocounters, s));
     C2_CUDA(cudaMemsetAsync(g.dirty, 1, ntiles, s));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     C2_CUDA(cudaEventCreate(&e0));
@@ -1176,6 +1294,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     const unsigned rgrid = (unsigned)((d.Hz + rb_r - 1) / rb_r * ntc);
     const Buckets2 bk2{g.bcount, g.bent, ntc};
     double dz32 = 0.0, all = 0.0;
+    long long counted[kSweepBatch] = {};
     for (;;) {
         bool settled = false;
         for (bool more = true; more;) {
@@ -1187,7 +1306,6 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                                    sweeps + kSweepBatch < 1000000
                                ? kSweepBatch
                                : 1;
-            C2_CUDA(cudaMemsetAsync(g.upd, 0, sizeof(long long) * nb, s));
             for (int b = 0; b < nb; b++) {
                 tp.upd = g.upd + b;
                 for (int p = 0; p < c; p++) {
@@ -1200,9 +1318,16 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                     launches++;
                 }
             }
-            long long u[kSweepBatch] = {};
-            C2_CUDA(cudaMemcpyAsync(u, g.upd, sizeof(long long) * nb, cudaMemcpyDeviceToHost, s));
+            // (the counters run on from batch to batch)
+            long long *const total = reinterpret_cast<long long *>(g.block.pin);
+            C2_CUDA(cudaMemcpyAsync(total, g.upd, sizeof(long long) * nb, cudaMemcpyDeviceToHost,
+                                    s));
             C2_CUDA(cudaStreamSynchronize(s));
+            long long u[kSweepBatch];
+            for (int b = 0; b < nb; b++) {
+                u[b] = total[b] - counted[b];
+                counted[b] = total[b];
+            }
             for (int b = 0; b < nb && more; b++) {
                 sweeps++;
                 updates += u[b];
@@ -1221,8 +1346,9 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                                               rb_r, (float)lambda, 1, bk2, g.red);
         C2_CUDA(cudaGetLastError());
         launches += 2;
-        unsigned long long red[8];
-        C2_CUDA(cudaMemcpyAsync(red, g.red, sizeof red, cudaMemcpyDeviceToHost, s));
+        unsigned long long *const red = g.block.pin;
+        C2_CUDA(cudaMemcpyAsync(red, g.red, sizeof(unsigned long long) * 8, cudaMemcpyDeviceToHost,
+                                s));
         C2_CUDA(cudaStreamSynchronize(s));
         std::memcpy(&dz32, &red[4], sizeof dz32);
         std::memcpy(&all, &red[3], sizeof all);
@@ -1244,11 +1370,13 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     sum_partials_kernel<<<1, 256, 0, s>>>(g.partial, ntile_o, lambda, g.E);
     C2_CUDA(cudaGetLastError());
     launches += 2;
-    double E = 0.0;
-    C2_CUDA(cudaMemcpyAsync(&E, g.E, sizeof E, cudaMemcpyDeviceToHost, s));
+    C2_CUDA(cudaMemcpyAsync(g.block.pin, g.E, sizeof(double), cudaMemcpyDeviceToHost, s));
     if (Z_out)
         C2_CUDA(copy_out(Z_out, g.Z, sizeof(float) * nz, s));
     C2_CUDA(cudaStreamSynchronize(s));
+    g.finished = true;
+    double E;
+    std::memcpy(&E, g.block.pin, sizeof E);
     float ms = 0.f;
     C2_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     cudaEventDestroy(e0);
@@ -1268,7 +1396,6 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
         stats->solve_ms = ms;
         stats->kernel_launches = launches;
     }
-    (void)dev;
     return converged ? CSC_OK : CSC_NOT_CONVERGED;
 }
 

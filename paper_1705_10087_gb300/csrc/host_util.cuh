@@ -85,6 +85,25 @@ inline cudaError_t copy_out(void *dst, const void *src, size_t bytes, cudaStream
                            s);
 }
 
+}  // namespace csc
+
+// Gives back the workspaces that finished calls left for the next ones (csc2d.cu).
+void csc_trim_workspaces();
+
+namespace csc {
+
+// cudaMalloc; when memory is short, once more after kept workspaces were given back.
+inline cudaError_t device_alloc(void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        csc_trim_workspaces();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 template <class T>
 cudaError_t grow(T **p, size_t *cap, size_t n)
 {
@@ -94,7 +113,7 @@ cudaError_t grow(T **p, size_t *cap, size_t n)
         cudaFree(*p);
     *p = nullptr;
     *cap = 0;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), sizeof(T) * (n ? n : 1));
+    cudaError_t e = device_alloc(reinterpret_cast<void **>(p), sizeof(T) * (n ? n : 1));
     if (e == cudaSuccess)
         *cap = n;
     return e;

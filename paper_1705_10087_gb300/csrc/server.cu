@@ -676,7 +676,7 @@ int csc_server_create(csc_server_t *sp, const csc_server_opts *opts)
     s->opts = o;
     cudaGetDevice(&s->device);
     void *base = nullptr;
-    cudaError_t e = cudaMalloc(&base, (size_t)o.hbm_budget_bytes);
+    cudaError_t e = device_alloc(&base, (size_t)o.hbm_budget_bytes);
     if (e != cudaSuccess) {
         delete s;
         return csc_record_error(CSC_ENOMEM, "csc_server_create: pool of %lld bytes: %s",

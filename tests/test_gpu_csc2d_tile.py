@@ -44,3 +44,39 @@ def test_tile_layout_edges_match_oracle(capi, K, P, h, w, H, W, M, N, u, frac, r
                                      lam, 1e-6, M=M, N=N, updates_per_visit=u, Z_out=Z)
     assert status == capi.CSC_OK and st["converged"] == 1, st
     assert_parity(Z.cpu().numpy(), E, ref["Z"], csc2d.objective(pb.D, pb.X, ref["Z"], lam))
+
+
+def test_calls_of_two_threads_share_no_workspace(capi):  # noqa: F811
+    # finished calls leave their device memory for later ones: calls that run at
+    # the same time on two streams must not meet in it, whatever their sizes
+    import threading
+
+    pbs = [synth.make_problem2d(K=3, P=1, h=4, w=5, H=40 + 30 * i, W=60 - 9 * i, rho=0.01,
+                                sigma=0.05, seed=20 + i) for i in range(2)]
+    lams = [0.1 * csc2d.lambda_max(pb.D, pb.X) for pb in pbs]
+
+    def solve(i, stream=None):
+        pb = pbs[i]
+        Z = torch.zeros((3, pb.X.shape[1] - 3, pb.X.shape[2] - 4), dtype=torch.float32,
+                        device="cuda")
+        torch.cuda.synchronize()
+        _, E, _ = capi.csc2d_solve(torch.from_numpy(pb.D).cuda(), torch.from_numpy(pb.X).cuda(),
+                                   lams[i], 1e-6, Z_out=Z, stream=stream)
+        return Z.cpu(), E
+
+    want = [solve(i) for i in range(2)]
+    bad = []
+
+    def run(i):
+        stream = torch.cuda.Stream()
+        for _ in range(6):
+            Z, E = solve(i, stream)
+            if not torch.equal(Z, want[i][0]) or E != want[i][1]:
+                bad.append(i)
+
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
