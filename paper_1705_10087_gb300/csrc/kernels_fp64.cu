@@ -7,6 +7,8 @@
 // reach its tile (compacted in a fixed order, so results are deterministic)
 // and every thread accumulates its outputs over that list in double-float
 // (pairs of floats with error-free transformations), combined in FP64.
+#include <type_traits>
+
 #include "csc_internal.cuh"
 #include "packed.cuh"
 
@@ -644,17 +646,94 @@ __global__ void __launch_bounds__(256, 4)
 }
 
 constexpr int kObjP = 8;    // channels accumulated per pass
+constexpr int kObjBatch = 16;  // atom rows of Z a warp loads at once (8: 1.5% slower calls)
 constexpr int kObjCap = 64;  // nonzeros of one 32-column bucket held in shared memory
 constexpr int kObjBuckets = kTile / 32 + (kMaxL - 1 + 31) / 32;
 
-// acc[q] += D[q L] z for the channels q < np of a pass (double-float)
-__device__ __forceinline__ void obj_add(float (&hi)[kObjP], float (&lo)[kObjP],
-                                        const float *__restrict__ Dk, int np, int L, float z)
+// Channels [p0, p0 + np) of one pass at sample t: (hi, lo) -= sum over the nonzeros
+// of the warp's buckets of D z, two channels per packed pair, in the buckets' order.
+// (A missing channel of the last pair, an entry past the end and one that does not
+// reach t all add 0 * 0, which changes neither hi nor lo.)
+//
+// Bound by the latency of entry -> coefficients -> sums: two entries are read by one
+// load and their coefficients together, and the sums take half the instructions of
+// one channel at a time.
+// P = 7, L = 64, K = 25, the whole kernel: 25 -> 20 us (T = 200000, 2% nonzeros
+// listed by a resync), 43 -> 33 us (the same, listed here), 485 -> 422 us (6.5 million
+// samples).  Four blocks per SM: at five the 48 registers spill.
+template <int NP>
+__device__ __forceinline__ void obj_pass(const uint2 (*ent)[kObjCap], const int *cnt, int j0,
+                                         int R, int64_t cb0, int64_t t, int64_t zhi,
+                                         const float *__restrict__ Dp, int np, int K, int P, int L,
+                                         const float *__restrict__ Z, int64_t ld,
+                                         const float *__restrict__ X, int64_t ldx, float &sq_h,
+                                         float &sq_l)
 {
+    unsigned long long hi[NP], lo[NP];
 #pragma unroll
-    for (int q = 0; q < kObjP; q++)
-        if (q < np)
-            df_add_prod(hi[q], lo[q], __ldg(Dk + q * L), z);
+    for (int q = 0; q < NP; q++)
+        hi[q] = lo[q] = 0ull;
+    const int PL = P * L;
+    for (int j = j0; j <= j0 + R; j++) {
+        const int n = cnt[j];
+        const int64_t cbj = cb0 + 32 * (int64_t)j;
+        if (n <= kObjCap) {
+            const int toff = (int)(t - cbj);
+#pragma unroll 1
+            for (int i = 0; i < n; i += 2) {
+                const uint4 e = *reinterpret_cast<const uint4 *>(&ent[j][i]);
+                const unsigned id[2] = {e.x, e.z};
+                float z[2] = {__uint_as_float(e.y), __uint_as_float(e.w)};
+                float a[2][2 * NP];
+#pragma unroll
+                for (int x = 0; x < 2; x++) {
+                    const int tau = toff - (int)(id[x] & 31u);
+                    const bool in = (x == 0 || i + 1 < n) && (unsigned)tau < (unsigned)L;
+                    z[x] = in ? z[x] : 0.f;
+                    const float *d = Dp + (in ? (int)(id[x] >> 5) * PL + tau : 0);
+#pragma unroll
+                    for (int q = 0; q < 2 * NP; q++, d += L)
+                        a[x][q] = in && q < np ? __ldg(d) : 0.f;
+                }
+#pragma unroll
+                for (int x = 0; x < 2; x++) {
+                    const unsigned long long z2 = pack2(z[x], z[x]), nz2 = pack2(-z[x], -z[x]);
+#pragma unroll
+                    for (int q = 0; q < NP; q++)
+                        df2_sub_prod(hi[q], lo[q], pack2(a[x][2 * q], a[x][2 * q + 1]), z2, nz2);
+                }
+            }
+        } else {
+            for (int k = 0; k < K; k++)
+                for (int jj = 0; jj < 32; jj++) {
+                    const int64_t tp = cbj + jj;
+                    const int tau = (int)(t - tp);
+                    if (tp < 0 || tp >= zhi || tau < 0 || tau >= L)
+                        continue;
+                    const float z = Z[(int64_t)k * ld + tp];
+                    if (z == 0.f)
+                        continue;
+                    const float *d = Dp + k * PL + tau;
+#pragma unroll
+                    for (int q = 0; q < NP; q++, d += 2 * L)
+                        df2_sub_prod(hi[q], lo[q],
+                                     pack2(2 * q < np ? __ldg(d) : 0.f,
+                                           2 * q + 1 < np ? __ldg(d + L) : 0.f),
+                                     pack2(z, z), pack2(-z, -z));
+                }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < NP; q++) {
+        float h0, h1, l0, l1;
+        unpack2(hi[q], h0, h1);
+        unpack2(lo[q], l0, l1);
+        // (the pairs hold minus the sums)
+        if (2 * q < np)
+            df_add_sq_residual(sq_h, sq_l, X[(int64_t)(2 * q) * ldx + t], -h0, -l0);
+        if (2 * q + 1 < np)
+            df_add_sq_residual(sq_h, sq_l, X[(int64_t)(2 * q + 1) * ldx + t], -h1, -l1);
+    }
 }
 
 // Tile b (kTile samples of one problem): partials[2b] = sum over its samples of
@@ -671,14 +750,14 @@ __device__ __forceinline__ void obj_add(float (&hi)[kObjP], float (&lo)[kObjP],
 // With lists (the buckets of the last resync, which saw this Z: same
 // entries in the same order) a bucket inside the problem is copied from the
 // resync tile starting at its first column, rtile_off[problem] + column / 32.
-__global__ void __launch_bounds__(kTile, 5)
+__global__ void __launch_bounds__(kTile, 4)
     objective_kernel(const float *__restrict__ D, const SigDesc *__restrict__ sigs, SigDesc one,
                      Tiles tiles, int K, int P, int L, const float *Zbase, const float *Zalt,
                      double *__restrict__ partials, NzLists lists,
                      const int64_t *__restrict__ rtile_off)
 {
     static_assert(kObjCap == kNzCap && kResyncCols == 32, "resync buckets serve the objective");
-    __shared__ uint2 ent[kObjBuckets][kObjCap];
+    __shared__ __align__(16) uint2 ent[kObjBuckets][kObjCap];  // (read two at a time)
     __shared__ int cnt[kObjBuckets];
     __shared__ double bsum[2][kTile / 32];
     const SigDesc sd = sigs ? sigs[tiles.sig[blockIdx.x]] : one;
@@ -710,14 +789,14 @@ __global__ void __launch_bounds__(kTile, 5)
         const int64_t col = cbj + lane;
         const bool in = col >= 0 && col < zhi;
         int base = 0;
-        for (int k0 = 0; k0 < K; k0 += kBucketBatch) {
-            // kBucketBatch rows loaded together: one memory round trip
-            float zv[kBucketBatch];
+        for (int k0 = 0; k0 < K; k0 += kObjBatch) {
+            // kObjBatch rows loaded together: one memory round trip
+            float zv[kObjBatch];
 #pragma unroll
-            for (int q = 0; q < kBucketBatch; q++)
+            for (int q = 0; q < kObjBatch; q++)
                 zv[q] = in && k0 + q < K ? Z[(int64_t)(k0 + q) * ld + col] : 0.f;
 #pragma unroll
-            for (int q = 0; q < kBucketBatch; q++) {
+            for (int q = 0; q < kObjBatch; q++) {
                 const float z = zv[q];
                 const unsigned m = __ballot_sync(0xffffffffu, z != 0.f);
                 if (z != 0.f) {
@@ -750,43 +829,20 @@ __global__ void __launch_bounds__(kTile, 5)
                     df_add(l1_h, l1_l, fabsf(Z[(int64_t)k * ld + col]));
         }
     }
-    for (int p0 = 0; p0 < P; p0 += kObjP) {
-        float acc_hi[kObjP], acc_lo[kObjP];
-#pragma unroll
-        for (int q = 0; q < kObjP; q++) {
-            acc_hi[q] = 0.f;
-            acc_lo[q] = 0.f;
-        }
-        if (t < c1) {
-            for (int j = warp; j <= warp + R; j++) {
-                const int n = cnt[j];
-                const int64_t cbj = cb0 + 32 * (int64_t)j;
-                if (n <= kObjCap) {
-                    for (int i = 0; i < n; i++) {
-                        const uint2 v = ent[j][i];
-                        const int tau = (int)(t - (cbj + (v.x & 31u)));
-                        if (tau >= 0 && tau < L)
-                            obj_add(acc_hi, acc_lo, D + ((int)(v.x >> 5) * P + p0) * L + tau,
-                                    P - p0, L, __uint_as_float(v.y));
-                    }
-                } else {
-                    for (int k = 0; k < K; k++)
-                        for (int jj = 0; jj < 32; jj++) {
-                            const int64_t tp = cbj + jj;
-                            const int tau = (int)(t - tp);
-                            if (tp < 0 || tp >= zhi || tau < 0 || tau >= L)
-                                continue;
-                            const float z = Z[(int64_t)k * ld + tp];
-                            if (z != 0.f)
-                                obj_add(acc_hi, acc_lo, D + (k * P + p0) * L + tau, P - p0, L, z);
-                        }
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < kObjP; q++)
-                if (p0 + q < P)
-                    df_add_sq_residual(sq_h, sq_l, sd.X[(int64_t)(p0 + q) * sd.ldx + t], acc_hi[q],
-                                       acc_lo[q]);
+    if (t < c1) {
+        auto pass = [&](auto pairs, int p0, int np) {
+            obj_pass<decltype(pairs)::value>(ent, cnt, warp, R, cb0, t, zhi, D + p0 * L, np, K, P,
+                                             L, Z, ld, sd.X + (int64_t)p0 * sd.ldx, sd.ldx, sq_h,
+                                             sq_l);
+        };
+        for (int p0 = 0; p0 < P; p0 += kObjP) {
+            const int np = P - p0 < kObjP ? P - p0 : kObjP;
+            if (np > 4)
+                pass(std::integral_constant<int, 4>{}, p0, np);
+            else if (np > 2)
+                pass(std::integral_constant<int, 2>{}, p0, np);
+            else
+                pass(std::integral_constant<int, 1>{}, p0, np);
         }
     }
     for (int off = 16; off > 0; off >>= 1) {
