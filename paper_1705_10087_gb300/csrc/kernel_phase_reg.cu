@@ -16,6 +16,16 @@ RegKernel reg_kernel(const PhaseConfig &cfg, bool dense)
     return by_nq[cfg.reg_nq - 1](cfg.block, cfg.reg_cb, dense);
 }
 
+// Blocks per SM of the form with more registers (96 a thread).  Launches of no more
+// blocks run it: nothing spills in the chain of updates (K = 25, P = 1, L = 200: T = 7396,
+// 18 segments, 21.3 -> 17.6 ms a solve; T = 93,992, 2.47 -> 2.20 ms).  Launches of more,
+// and those that drain a queue, run the one with more blocks per SM (T = 5,000,000: 26.6 ms
+// with one block per SM, 22.4 with two).
+int roomy_blocks(int block)
+{
+    return block <= 160 ? 4 : block <= 288 ? 2 : 1;
+}
+
 int sm_count()
 {
     int dev = 0, nsm = 1;
@@ -59,8 +69,8 @@ bool phase_reg_config(int K, int L, int w_max, PhaseConfig *cfg)
 cudaError_t launch_phase_reg(const PhaseParams &pp, const PhaseConfig &cfg, int grid, bool drain,
                              cudaStream_t s)
 {
-    // (at most 4 blocks per SM: the form with more registers)
-    RegKernel kern = reg_kernel(cfg, drain || grid > 4 * sm_count());
+    // (all blocks resident with more registers: the form with more registers)
+    RegKernel kern = reg_kernel(cfg, drain || grid > roomy_blocks(cfg.block) * sm_count());
     if (!kern || cfg.reg_cb < 2 * pp.L - 1 || pp.w_max > cfg.reg_ns * cfg.reg_cb ||
         (cfg.block - 32) / cfg.reg_cb * cfg.reg_nq * 4 < pp.K)
         return cudaErrorInvalidConfiguration;

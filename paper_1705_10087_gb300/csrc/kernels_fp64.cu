@@ -658,7 +658,7 @@ constexpr int kObjBuckets = kTile / 32 + (kMaxL - 1 + 31) / 32;
 // Bound by the latency of entry -> coefficients -> sums: two entries are read by one
 // load and their coefficients together, and the sums take half the instructions of
 // one channel at a time.
-// P = 7, L = 64, K = 25, the whole kernel: 25 -> 20 us (T = 200000, 2% nonzeros
+// P = 7, L = 64, K = 25, the whole kernel: 25 -> 20 us (T = 200000, the nonzeros
 // listed by a resync), 43 -> 33 us (the same, listed here), 485 -> 422 us (6.5 million
 // samples).  Four blocks per SM: at five the 48 registers spill.
 template <int NP>

@@ -551,16 +551,16 @@ __global__ void __launch_bounds__(MAXT, MINB)
 // The instantiation for blocks of `block` threads (registers: at most 65536 /
 // (threads x blocks per SM)).  dense: more segments than fit at once, so the
 // blocks per SM count; else a segment's chain of
-// updates counts.  One group of atoms (K <= 32) has a form for every NQ, so no
+// updates counts (launch_phase_reg has the line).  One group of atoms (K <= 32) has a form for every NQ, so no
 // quad is padding; with more groups the last one may be short (TAIL).
 template <int NQ, bool TAIL>
 RegKernel by_block(int block, bool dense)
 {
     if (block <= 160)
         return dense ? phase_reg_kernel<NQ, TAIL, 160, 5> : phase_reg_kernel<NQ, TAIL, 160, 4>;
-    if (block <= 288)
+    if (dense && block <= 288)
         return phase_reg_kernel<NQ, TAIL, 288, 3>;
-    if (block <= 448)
+    if (dense && block <= 448)
         return phase_reg_kernel<NQ, TAIL, 448, 2>;
     return phase_reg_kernel<NQ, TAIL, 544, 1>;
 }

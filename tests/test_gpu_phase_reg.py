@@ -46,3 +46,19 @@ def test_phase_layout_edges_match_oracle(capi, K, P, L, T, M, u, frac):  # noqa:
     r = gpu_solve(capi, pb, lam, 1e-6, M=M, u=u)
     assert r["status"] == 0 and r["stats"]["segments"] == M, r["stats"]
     assert_parity(r["Z"], r["E"], ref["Z"], oracle.objective(pb.D, pb.X, ref["Z"], lam))
+
+
+@pytest.mark.parametrize("K,P,L,T,M", [
+    (4, 4, 70, 20_000, 100),   # 192-thread blocks, all resident in the form with more registers
+    (4, 4, 70, 88_000, 632),   # and more than that
+    (4, 2, 150, 30_000, 90),   # 352-thread blocks
+    (4, 2, 150, 93_000, 306),
+])
+def test_few_and_many_segments_match_oracle(capi, K, P, L, T, M):  # noqa: F811
+    pb = synth.make_problem(K=K, P=P, L=L, T=T, rho=0.001, sigma=0.1, seed=K + L)
+    lam = 0.1 * oracle.lambda_max(pb.D, pb.X)
+    ref = oracle.locally_greedy_cd(pb.D, pb.X, lam, 1e-10, M=M, mode="phase")
+    assert ref["converged"]
+    r = gpu_solve(capi, pb, lam, 1e-6, M=M, u=24)
+    assert r["status"] == 0 and r["stats"]["segments"] == M, r["stats"]
+    assert_parity(r["Z"], r["E"], ref["Z"], oracle.objective(pb.D, pb.X, ref["Z"], lam))
