@@ -170,7 +170,8 @@ def phase_profile():
     import hashlib
     try:
         text = open(os.path.join(ROOT, "profiles", f"phase_kernel_{WORKLOAD}.md")).read()
-        src = open(os.path.join(ROOT, "paper_1705_10087_gb300", "csrc", "kernel_phase.cu"), "rb").read()
+        src = open(os.path.join(ROOT, "paper_1705_10087_gb300", "csrc",
+                                "phase_reg_impl.cuh"), "rb").read()
     except OSError:
         return {}
     fields = dict(ln.split(":", 1) for ln in text.splitlines()
