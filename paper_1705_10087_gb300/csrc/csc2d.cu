@@ -940,12 +940,13 @@ int auto_bands(int64_t Hz, int h)
 // Workspaces kept between calls: a finished call leaves its device block (and 512
 // bytes of pinned memory for read-backs) for the next one, because cudaMalloc,
 // cudaFree and the synchronisation they imply took 0.3 to 0.4 ms of a call.  At most
-// kKeep2 bytes are kept in all (the oldest go first; larger blocks are freed at
-// once), and all of them are given back when an allocation of this library fails
+// kKeep2 bytes in kKept2 blocks are kept in all (the oldest go first; larger blocks
+// are freed at once; the list itself allocates nothing), and all of them are given back when an allocation of this library fails
 // (csc_trim_workspaces).  A block belongs to one call at a time and is only put
 // back after its stream was waited for, so threads and streams never share one.
 constexpr size_t kKeep2 = (size_t)64 << 20;
 constexpr size_t kPin2 = 512;
+constexpr int kKept2 = 16;
 struct Block2 {
     void *dev = nullptr;
     size_t cap = 0;
@@ -954,12 +955,21 @@ struct Block2 {
 };
 struct Kept2 {
     std::mutex mutex;
-    std::vector<Block2> blocks;  // oldest first
+    Block2 blocks[kKept2];  // oldest first
+    int n = 0;
+
+    Block2 remove(int i)
+    {
+        const Block2 b = blocks[i];
+        for (n--; i < n; i++)
+            blocks[i] = blocks[i + 1];
+        return b;
+    }
 };
 Kept2 &kept2()
 {
-    static Kept2 *k = new Kept2;  // (never destroyed: no order at exit to mind)
-    return *k;
+    static Kept2 k;
+    return k;
 }
 
 void free_block2(const Block2 &b)
@@ -975,12 +985,12 @@ cudaError_t take_block2(int device, size_t bytes, Block2 *out)
     {
         Kept2 &k = kept2();
         std::lock_guard<std::mutex> lock(k.mutex);
-        for (size_t i = 0; i < k.blocks.size(); i++) {
+        for (int i = 0; i < k.n; i++) {
             const Block2 b = k.blocks[i];
             // (no more than four times what is asked for)
             if (b.device != device || b.cap < bytes || b.cap / 4 > bytes + (1 << 20))
                 continue;
-            k.blocks.erase(k.blocks.begin() + i);
+            k.remove(i);
             // memory that a device reset has taken away is no block
             cudaPointerAttributes at;
             if (cudaPointerGetAttributes(&at, b.dev) != cudaSuccess ||
@@ -1009,24 +1019,24 @@ cudaError_t take_block2(int device, size_t bytes, Block2 *out)
 
 void keep_block2(const Block2 &b)
 {
-    std::vector<Block2> drop;
+    Block2 drop[kKept2 + 1];
+    int nd = 0;
     if (b.cap > kKeep2) {
-        drop.push_back(b);
+        drop[nd++] = b;
     } else {
         Kept2 &k = kept2();
         std::lock_guard<std::mutex> lock(k.mutex);
-        k.blocks.push_back(b);
-        size_t total = 0;
-        for (const Block2 &x : k.blocks)
-            total += x.cap;
-        while (total > kKeep2) {
-            total -= k.blocks.front().cap;
-            drop.push_back(k.blocks.front());
-            k.blocks.erase(k.blocks.begin());
+        size_t total = b.cap;
+        for (int i = 0; i < k.n; i++)
+            total += k.blocks[i].cap;
+        while (k.n && (total > kKeep2 || k.n == kKept2)) {
+            total -= k.blocks[0].cap;
+            drop[nd++] = k.remove(0);
         }
+        k.blocks[k.n++] = b;
     }
-    for (const Block2 &x : drop)
-        free_block2(x);
+    for (int i = 0; i < nd; i++)
+        free_block2(drop[i]);
 }
 
 // Device buffers of one csc2d_solve call, carved from one block.
@@ -1059,14 +1069,16 @@ struct Dev2 {
 
 void csc_trim_workspaces()
 {
-    std::vector<Block2> drop;
+    Block2 drop[kKept2];
+    int nd = 0;
     {
         Kept2 &k = kept2();
         std::lock_guard<std::mutex> lock(k.mutex);
-        drop.swap(k.blocks);
+        while (k.n)
+            drop[nd++] = k.remove(k.n - 1);
     }
-    for (const Block2 &x : drop)
-        free_block2(x);
+    for (int i = 0; i < nd; i++)
+        free_block2(drop[i]);
 }
 
 extern "C" {
