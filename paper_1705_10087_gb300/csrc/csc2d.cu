@@ -1164,7 +1164,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
     const int64_t max_ext = (hmax + 2 * h - 2) * (wmax + 2 * w - 2);
     const size_t reg_smem = tile_reg_smem(nq, max_ext, max_pos);
     const int64_t nslots = ((hmax + 4 * h - 4) / (2 * h - 1)) * ((wmax + 4 * w - 4) / (2 * w - 1));
-    const bool reg = K <= 32 && A <= 512 && reg_smem <= (size_t)kMaxSmem - 4096 && nslots <= 32 &&
+    const bool reg = K <= 32 && A <= 512 && reg_smem <= (size_t)kTileRegSmem && nslots <= 32 &&
                      bits(hmax - 1) + bits(wmax - 1) <= 24;
     // a tile's r and Z are staged in shared memory when they fit
     const bool stage = TileLayout(K, (int)max_pos, true).total <= (size_t)kMaxSmem;
@@ -1278,8 +1278,7 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
         launches += 2;
     }
     auto tile_fn = reg ? tile_reg_fn(K, block) : stage ? tile_kernel<true> : tile_kernel<false>;
-    C2_CUDA(cudaFuncSetAttribute(tile_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
+    C2_CUDA(allow_smem(tile_fn, reg ? kTileRegSmem : kMaxSmem));
     TileParams tp;
     tp.r = g.r;
     tp.Z = g.Z;

@@ -26,6 +26,7 @@ namespace {
 using namespace csc;
 
 constexpr int kPosWarps = 16;  // position warps of a block at most (and the active warp)
+constexpr int kTileRegSmem = kMaxSmem - 4096;  // dynamic shared memory at most (static: 3 KB)
 
 // Shared memory (bytes): ext positions of NQ | 1 quads (tile and halo), and per tile
 // position a key and the bits of its listed and unlisted nonzeros.

@@ -206,6 +206,17 @@ struct PhaseParams {
     int *queue;
 };
 
+// Lets a kernel ask for up to `most` bytes of dynamic shared memory.  The limit
+// belongs to the function on its device, not to a launch: a call that set it to
+// its own need would lower it between another thread's setting and launch, which
+// is then refused.  So all calls set one value per kernel, the most that the rule
+// of its dispatch admits.
+template <class Kernel>
+inline cudaError_t allow_smem(Kernel *kern, size_t most = kMaxSmem)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 struct PhaseConfig {
     int block = 0;
     size_t smem = 0;

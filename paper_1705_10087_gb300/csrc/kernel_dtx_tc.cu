@@ -649,8 +649,7 @@ cudaError_t launch_dtx_tc(const float *D, const float *X, int K, int P, int L, i
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     // max_per_sm: tensor-memory columns allow at most 512 / (columns per CTA)
     auto go = [&](auto kern, int max_per_sm) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = allow_smem(kern);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (e != cudaSuccess)

@@ -1045,8 +1045,7 @@ cudaError_t launch_phase(const PhaseParams &pp, const PhaseConfig &cfg, int acti
     if (e != cudaSuccess)
         return e;
     e = dispatch<PerSegment>(cfg, pp.K, [&](auto kern) -> cudaError_t {
-        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)cfg.smem);
+        cudaError_t r = allow_smem(kern);
         if (r != cudaSuccess)
             return r;
         kern<<<active, cfg.block, cfg.smem, s>>>(pp);
@@ -1065,7 +1064,7 @@ int phase_resident_blocks(const PhaseConfig &cfg, int K)
     if (cfg.reg_nq > 0)
         return nsm * std::max(1, phase_reg_blocks_per_sm(cfg));
     dispatch<Drain>(cfg, K, [&](auto kern) -> cudaError_t {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.smem);
+        allow_smem(kern);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, cfg.block, cfg.smem);
         return cudaSuccess;
     });
@@ -1095,8 +1094,7 @@ cudaError_t launch_phase_drain(const PhaseParams &pp, const PhaseConfig &cfg, in
     if (cfg.reg_nq > 0)
         return launch_phase_reg(pp, cfg, grid, true, s);
     e = dispatch<Drain>(cfg, pp.K, [&](auto kern) -> cudaError_t {
-        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)cfg.smem);
+        cudaError_t r = allow_smem(kern);
         if (r != cudaSuccess)
             return r;
         kern<<<grid, cfg.block, cfg.smem, s>>>(pp);

@@ -53,7 +53,7 @@ bool phase_reg_config(int K, int L, int w_max, PhaseConfig *cfg)
         // two bits of the changed mask are the halo's)
         const int ns = (w_max + cb - 1) / cb;
         const size_t smem = phase_reg_smem(nq, groups, L, w_max);
-        if (groups * cb > 512 || ns > 30 || smem > (size_t)kMaxSmem - 8192)
+        if (groups * cb > 512 || ns > 30 || smem > (size_t)kPhaseRegSmem)
             continue;
         cfg->reg_nq = nq;
         cfg->reg_ns = ns;
@@ -74,8 +74,7 @@ cudaError_t launch_phase_reg(const PhaseParams &pp, const PhaseConfig &cfg, int 
     if (!kern || cfg.reg_cb < 2 * pp.L - 1 || pp.w_max > cfg.reg_ns * cfg.reg_cb ||
         (cfg.block - 32) / cfg.reg_cb * cfg.reg_nq * 4 < pp.K)
         return cudaErrorInvalidConfiguration;
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.smem);
+    const cudaError_t e = allow_smem(kern, kPhaseRegSmem);
     if (e != cudaSuccess)
         return e;
     kern<<<grid, cfg.block, cfg.smem, s>>>(pp, cfg.reg_cb, drain ? 1 : 0);
@@ -87,7 +86,7 @@ int phase_reg_blocks_per_sm(const PhaseConfig &cfg)
     int per_sm = 1;
     RegKernel kern = reg_kernel(cfg, true);
     if (kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.smem);
+        allow_smem(kern, kPhaseRegSmem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, cfg.block, cfg.smem);
     }
     return per_sm;

@@ -272,8 +272,7 @@ cudaError_t launch_dtx(const float *D, const float *X, int K, int P, int L, int6
         sizeof(float) * ((size_t)P * (kDtxTile + L8 + 4) + (size_t)kDtxAtoms * P * L8);
     if (smem > (size_t)kMaxSmem)
         return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(dtx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const cudaError_t e = allow_smem(dtx_kernel);
     if (e != cudaSuccess)
         return e;
     const int64_t Tz = T - L + 1;
