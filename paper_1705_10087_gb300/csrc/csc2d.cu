@@ -1270,6 +1270,8 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
         dtd2d_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(g.D, d, KQ,
                                                                                        g.Ct, g.norms);
         C2_CUDA(cudaGetLastError());
+        // ((2h-1)(2w-1) <= kMaxWin allows h w <= 2048, one-row atoms of 2048 columns)
+        C2_CUDA(allow_smem(dtx2d_kernel, sizeof(float) * kAtoms2 * kMaxWin / 2));
         dtx2d_kernel<<<dim3((unsigned)((d.Hz * d.Wz + 255) / 256),
                             (unsigned)((K + kAtoms2 - 1) / kAtoms2)),
                        256, sizeof(float) * kAtoms2 * h * w, s>>>(g.D, g.X, d, g.beta0, g.r, g.Z,
