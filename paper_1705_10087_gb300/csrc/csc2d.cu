@@ -30,10 +30,13 @@
 // barrier) -> update -> re-evaluation of the window's positions, writing the
 // window positions outside its tile (idle neighbours) with atomicAdd and each new
 // Z value to global memory when it is applied.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "csc2d.h"
@@ -941,9 +944,17 @@ int auto_bands(int64_t Hz, int h)
 // bytes of pinned memory for read-backs) for the next one, because cudaMalloc,
 // cudaFree and the synchronisation they imply took 0.3 to 0.4 ms of a call.  At most
 // kKeep2 bytes in kKept2 blocks are kept in all (the oldest go first; larger blocks
-// are freed at once; the list itself allocates nothing), and all of them are given back when an allocation of this library fails
-// (csc_trim_workspaces).  A block belongs to one call at a time and is only put
-// back after its stream was waited for, so threads and streams never share one.
+// are freed at once; the list itself allocates nothing), and all of them are given
+// back when an allocation of this library fails (csc_trim_workspaces).  A block
+// belongs to one call at a time and is only put back after its stream was waited
+// for, so threads and streams never share one.
+//
+// A block lives as long as its context.  A device reset ends the primary context
+// without a word to this library, and an allocation after it can get the very
+// address of a kept block: so a block carries the id of its context, which the
+// driver never gives twice.  It is used, and freed, under that id only, and
+// forgotten when the device's primary context has another one.  (The blocks of other
+// contexts, whose end cannot be seen from here, are not kept.)
 constexpr size_t kKeep2 = (size_t)64 << 20;
 constexpr size_t kPin2 = 512;
 constexpr int kKept2 = 16;
@@ -951,6 +962,7 @@ struct Block2 {
     void *dev = nullptr;
     size_t cap = 0;
     int device = 0;
+    unsigned long long ctx = 0;  // id of its context (0: unknown)
     unsigned long long *pin = nullptr;
 };
 struct Kept2 {
@@ -972,37 +984,118 @@ Kept2 &kept2()
     return k;
 }
 
+// The driver's context calls (ok: all of them are there).
+struct Driver2 {
+    decltype(&cuDeviceGet) device = nullptr;
+    decltype(&cuCtxGetId) id = nullptr;
+    decltype(&cuCtxPushCurrent) push = nullptr;
+    decltype(&cuCtxPopCurrent) pop = nullptr;
+    decltype(&cuDevicePrimaryCtxGetState) state = nullptr;
+    decltype(&cuDevicePrimaryCtxRetain) retain = nullptr;
+    decltype(&cuDevicePrimaryCtxRelease) release = nullptr;
+    bool ok = true;
+
+    Driver2()
+    {
+        auto find = [this](auto &fn, const char *name) {
+            void *p = nullptr;
+            cudaDriverEntryPointQueryResult found;
+            ok = ok &&
+                 cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &found) ==
+                     cudaSuccess &&
+                 p;
+            fn = reinterpret_cast<std::decay_t<decltype(fn)>>(p);
+        };
+        find(device, "cuDeviceGet");
+        find(id, "cuCtxGetId");
+        find(push, "cuCtxPushCurrent");
+        find(pop, "cuCtxPopCurrent");
+        find(state, "cuDevicePrimaryCtxGetState");
+        find(retain, "cuDevicePrimaryCtxRetain");
+        find(release, "cuDevicePrimaryCtxRelease");
+        cudaGetLastError();
+    }
+};
+const Driver2 &driver2()
+{
+    static const Driver2 d;
+    return d;
+}
+
+// Id of the calling thread's context, 0 when it is not known.
+unsigned long long context_id()
+{
+    const Driver2 &d = driver2();
+    unsigned long long id = 0;
+    if (!d.ok || d.id(nullptr, &id) == CUDA_SUCCESS)
+        return id;
+    cudaFree(nullptr);  // none yet, or gone with a reset: the runtime makes one
+    cudaGetLastError();
+    return d.id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// A device's primary context, held for a scope (id 0: there is none).
+struct Primary2 {
+    CUdevice dev = 0;
+    CUcontext ctx = nullptr;
+    unsigned long long id = 0;
+    explicit Primary2(int device)
+    {
+        const Driver2 &d = driver2();
+        unsigned flags = 0;
+        int active = 0;
+        if (!d.ok || d.device(&dev, device) != CUDA_SUCCESS ||
+            d.state(dev, &flags, &active) != CUDA_SUCCESS || !active)
+            return;
+        if (d.retain(&ctx, dev) != CUDA_SUCCESS)
+            ctx = nullptr;
+        else if (d.id(ctx, &id) != CUDA_SUCCESS)
+            id = 0;
+    }
+    ~Primary2()
+    {
+        if (ctx)
+            driver2().release(dev);
+    }
+    Primary2(const Primary2 &) = delete;
+    Primary2 &operator=(const Primary2 &) = delete;
+};
+
+// Frees a block of the current context.
 void free_block2(const Block2 &b)
 {
-    csc::DeviceGuard guard(b.device);
     cudaFree(b.dev);
     cudaFreeHost(b.pin);
     cudaGetLastError();
 }
 
+// Frees a block that was kept, unless its context has ended.
+void drop_block2(const Block2 &b)
+{
+    const Primary2 p(b.device);
+    if (p.id == 0 || p.id != b.ctx || driver2().push(p.ctx) != CUDA_SUCCESS)
+        return;
+    free_block2(b);
+    CUcontext popped;
+    driver2().pop(&popped);
+}
+
 cudaError_t take_block2(int device, size_t bytes, Block2 *out)
 {
-    {
+    Block2 b;
+    b.ctx = context_id();
+    if (b.ctx) {
         Kept2 &k = kept2();
         std::lock_guard<std::mutex> lock(k.mutex);
         for (int i = 0; i < k.n; i++) {
-            const Block2 b = k.blocks[i];
+            const Block2 &have = k.blocks[i];
             // (no more than four times what is asked for)
-            if (b.device != device || b.cap < bytes || b.cap / 4 > bytes + (1 << 20))
-                continue;
-            k.remove(i);
-            // memory that a device reset has taken away is no block
-            cudaPointerAttributes at;
-            if (cudaPointerGetAttributes(&at, b.dev) != cudaSuccess ||
-                at.type != cudaMemoryTypeDevice || at.device != device) {
-                cudaGetLastError();
-                break;
+            if (have.ctx == b.ctx && have.cap >= bytes && have.cap / 4 <= bytes + (1 << 20)) {
+                *out = k.remove(i);
+                return cudaSuccess;
             }
-            *out = b;
-            return cudaSuccess;
         }
     }
-    Block2 b;
     b.device = device;
     b.cap = bytes;
     cudaError_t e = csc::device_alloc(&b.dev, bytes);
@@ -1019,16 +1112,23 @@ cudaError_t take_block2(int device, size_t bytes, Block2 *out)
 
 void keep_block2(const Block2 &b)
 {
-    Block2 drop[kKept2 + 1];
+    const Primary2 p(b.device);
+    if (b.cap > kKeep2 || p.id == 0 || p.id != b.ctx) {
+        free_block2(b);
+        return;
+    }
+    Block2 drop[kKept2];
     int nd = 0;
-    if (b.cap > kKeep2) {
-        drop[nd++] = b;
-    } else {
+    {
         Kept2 &k = kept2();
         std::lock_guard<std::mutex> lock(k.mutex);
         size_t total = b.cap;
-        for (int i = 0; i < k.n; i++)
-            total += k.blocks[i].cap;
+        for (int i = k.n - 1; i >= 0; i--) {
+            if (k.blocks[i].device == b.device && k.blocks[i].ctx != b.ctx)
+                k.remove(i);  // (went with an earlier primary context)
+            else
+                total += k.blocks[i].cap;
+        }
         while (k.n && (total > kKeep2 || k.n == kKept2)) {
             total -= k.blocks[0].cap;
             drop[nd++] = k.remove(0);
@@ -1036,7 +1136,7 @@ void keep_block2(const Block2 &b)
         k.blocks[k.n++] = b;
     }
     for (int i = 0; i < nd; i++)
-        free_block2(drop[i]);
+        drop_block2(drop[i]);
 }
 
 // Device buffers of one csc2d_solve call, carved from one block.
@@ -1078,7 +1178,7 @@ void csc_trim_workspaces()
             drop[nd++] = k.remove(k.n - 1);
     }
     for (int i = 0; i < nd; i++)
-        free_block2(drop[i]);
+        drop_block2(drop[i]);
 }
 
 extern "C" {
