@@ -64,7 +64,8 @@ int csc2d_plan(int64_t Hz, int h, int M, int *M_out, int *phases, int64_t *start
  * objective.  The state is float32 (the same numerics as csc_solve: the
  * float32 resolution floor applies).  The call takes its device memory on the
  * current device; up to 64 MiB of it in all stays with the library for later
- * calls (given back when an allocation of the library fails).
+ * calls (given back by csc2d_trim, and when an allocation of the library fails;
+ * a device reset ends it).
  *   D [K][P][h][w], X [P][H][W]: host or device, caller-owned
  *   1 <= K <= 64, P <= 64, K (2h-1) <= 2048, (2h-1)(2w-1) <= 4096; a tile's
  *   positions times 20 bytes must fit shared memory (about 226 KB; its r and
@@ -83,6 +84,11 @@ int csc2d_solve(const float *D, int K, int P, int h, int w, const float *X, int6
                 int64_t W, double lambda, double tol, int64_t max_updates, int M, int N,
                 int updates_per_visit, float *Z_out, double *objective, csc2d_stats *stats,
                 void *stream);
+
+/* Gives back, on all devices, the memory that finished csc2d_solve calls left for
+ * later ones.  At any time and from any thread: calls in progress keep theirs.
+ * Returns CSC_OK. */
+int csc2d_trim(void);
 
 #ifdef __cplusplus
 }

@@ -670,3 +670,8 @@ def csc2d_solve(D, X, lam: float, tol: float, max_updates: int = 1 << 62, M: int
                                        int(updates_per_visit), _ptr(Z_out, True),
                                        ctypes.byref(obj), ctypes.byref(st), _stream(stream)))
     return status, obj.value, st.as_dict()
+
+
+def csc2d_trim() -> None:
+    """Gives back the device memory that finished csc2d_solve calls left for later ones."""
+    _check(load().csc2d_trim())

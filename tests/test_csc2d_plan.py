@@ -27,3 +27,8 @@ def test_band_plan_automatic_and_rejects(lib):
     assert min(b - a for a, b in zip(starts[:-1], starts[1:])) >= 2 * 8 - 2 and c == 2
     with pytest.raises(capi.CscError):
         capi.csc2d_plan(10, 4, 11)
+
+
+def test_trim_without_a_device_does_nothing():
+    build.build()
+    capi.csc2d_trim()

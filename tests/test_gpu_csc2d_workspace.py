@@ -1,5 +1,5 @@
-"""The device memory that finished csc2d_solve calls keep for later ones: what becomes
-of it when the device is reset between two calls."""
+"""The device memory that finished csc2d_solve calls keep for later ones: how it is given
+back, and what becomes of it when the device is reset between two calls."""
 import os
 import subprocess
 import sys
@@ -71,3 +71,23 @@ def test_a_device_reset_ends_the_kept_memory(capi):  # noqa: F811
     if r.returncode == 77:
         pytest.skip("no CUDA runtime library to reset the device with")
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_trim_gives_the_kept_memory_back(capi):  # noqa: F811
+    D = torch.randn((8, 1, 8, 8), device="cuda")
+    X = torch.randn((1, 512, 512), device="cuda")
+    need = 3 * 4 * 8 * 505 * 505  # beta0, r and Z alone
+
+    def solve_and_free_bytes():
+        capi.csc2d_solve(D, X, 1e6, 1e-6)  # (lambda above lambda_max: Z = 0)
+        return torch.cuda.mem_get_info()[0]
+
+    solve_and_free_bytes()  # (kernels loaded)
+    capi.csc2d_trim()
+    empty = torch.cuda.mem_get_info()[0]
+    for _ in range(2):
+        assert solve_and_free_bytes() <= empty - need
+        capi.csc2d_trim()
+        assert torch.cuda.mem_get_info()[0] == empty
+    capi.csc2d_trim()  # (nothing left: no effect)
+    assert torch.cuda.mem_get_info()[0] == empty
