@@ -721,8 +721,9 @@ int csc_init_batch(csc_handle_t h, const float *X, const int64_t *T, int n, cons
         CSC_CUDA(cudaEventCreate(&h->ev_i1));
     }
     // a cold start (Z = 0) has r = beta0: the kernel writes both and zeroes Z;
-    // the tensor-core kernel also, for a batch, takes the per-signal maxima (the kernel's overall maximum also covers the columns between
-    // signals, which belong to no problem)
+    // the tensor-core kernel also, for a batch, takes the per-signal maxima (the
+    // kernel's overall maximum also covers the columns between signals, which belong
+    // to no problem)
     Dtx0Extras ex;
     if (!Z0)
         ex.z_out = h->Z;

@@ -417,8 +417,12 @@ __global__ void __launch_bounds__(MAXT, MINB) tile_reg_kernel(TileParams tp)
 
 using TileKernel = void (*)(TileParams);
 
-// registers: 65536 / (threads x blocks per SM) at most; three blocks of 288
-// threads hold the 324 co-active tiles of a 512 x 512 image with 8 x 8 atoms
+// registers: 65536 / (threads x blocks per SM) at most.  Blocks of 161 to 288 threads
+// (windows of 129 to 256 positions): three per SM, so that 456 tiles run at once, at 72
+// registers and with spills beyond 8 atoms.  With two per SM (96 registers) many tiles
+// are slower, few are faster, calls with 8 x 8 atoms: 1024 x 1024 with K = 8 and K = 2
+// 4.18 and 1.21 ms instead of 4.02 and 1.14; 512 x 512, K = 8 2.52 instead of 2.58;
+// 256 x 256 with K = 16 7.9 instead of 10.1.
 template <int NQ>
 TileKernel tile_reg_block(int block)
 {

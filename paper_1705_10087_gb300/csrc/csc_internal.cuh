@@ -221,14 +221,15 @@ struct PhaseConfig {
     int block = 0;
     size_t smem = 0;
     bool tile_in_smem = false;
-    // the register form (kernel_phase_reg.cu) when reg_nq > 0: float4 groups of
+    // the thread-private form (kernel_phase_reg.cu) when reg_nq > 0: float4 groups of
     // atoms per thread, columns per thread, threads per group of atoms
     int reg_nq = 0, reg_ns = 0, reg_cb = 0;
 };
 
 // w_max: widest segment of the plan; threads_per_segment: 32 = one warp per
 // segment where eligible (K = 25, 2L-1 <= 128, the tile fits shared memory),
-// otherwise (and for 0) a block of 128, 512 or 1024 threads.
+// otherwise (and for 0) a block: the thread-private form where phase_reg_config
+// accepts (64 to 544 threads), else phase_kernel with 128, 512 or 1024.
 PhaseConfig phase_config(int K, int L, int w_max, int threads_per_segment);
 bool phase_warp_eligible(int K, int L, int w_max);
 // active = number of segments in pp.phase_list (the grid size).

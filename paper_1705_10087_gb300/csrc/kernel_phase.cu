@@ -39,9 +39,11 @@
 // since is clean and is skipped: r and Z on it have not changed.
 //
 // Segments that fit run the form of phase_reg_impl.cuh (same updates, same bits, 1.4
-// to 4.8 times the speed); this one runs what phase_reg_config refuses: segments too
-// wide for shared memory, windows of more than 255 columns with K > 32, L > 256.  The
-// warp form (threads_per_segment = 32) is here too.
+// to 4.8 times the speed); this one runs what phase_reg_config refuses: more than 512
+// threads, ceil(K / 32) groups of atoms times 2L-1 rounded up to 32 (L > 256 at
+// K <= 32, L > 128 at K = 33 .. 64, L > 80 at K = 65 .. 96, ...), and segments too
+// wide for shared memory or for 30 columns per thread.  The warp form
+// (threads_per_segment = 32) is here too.
 #include <algorithm>
 #include <type_traits>
 
@@ -983,7 +985,7 @@ cudaError_t dispatch(const PhaseConfig &cfg, int K, F &&f)
         return f(Sel<true, 32, 25>::fn());
     // the workloads' atom counts (25 and 64) are compiled with K fixed (their
     // staged form only where phase_reg_config refuses what would fit: K = 64 with
-    // windows of more than 255 columns)
+    // L > 128)
     if (cfg.block == 128) {
         if (K == 25)
             return f(Sel<false, 128, 25>::fn());

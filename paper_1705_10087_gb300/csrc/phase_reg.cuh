@@ -1,5 +1,5 @@
-// The phase kernel with r in registers (kernel_phase_reg.cu), chosen by
-// phase_config (kernel_phase.cu) and launched through launch_phase and
+// The phase kernel with thread-private r in shared memory (phase_reg_impl.cuh), chosen
+// by phase_config (kernel_phase.cu) and launched through launch_phase and
 // launch_phase_drain.
 #pragma once
 
@@ -7,8 +7,8 @@
 
 namespace csc {
 
-// Fills cfg (reg_nq > 0) when the registers of a block hold a segment of w_max
-// columns; false where the shared-memory form must run.
+// Fills cfg (reg_nq > 0) when a block's threads and shared memory hold a segment of
+// w_max columns; false where phase_kernel must run.
 bool phase_reg_config(int K, int L, int w_max, PhaseConfig *cfg);
 cudaError_t launch_phase_reg(const PhaseParams &pp, const PhaseConfig &cfg, int grid, bool drain,
                              cudaStream_t s);

@@ -569,9 +569,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
 
 // The instantiation for blocks of `block` threads (registers: at most 65536 /
 // (threads x blocks per SM)).  dense: more segments than fit at once, so the
-// blocks per SM count; else a segment's chain of
-// updates counts (launch_phase_reg has the line).  One group of atoms (K <= 32) has a form for every NQ, so no
-// quad is padding; with more groups the last one may be short (TAIL).
+// blocks per SM count; else a segment's chain of updates counts (launch_phase_reg has
+// the line).  One group of atoms (K <= 32) has a form for every NQ, so no quad is
+// padding; with more groups the last one may be short (TAIL).
 template <int NQ, bool TAIL>
 RegKernel by_block(int block, bool dense)
 {
