@@ -163,20 +163,35 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def phase_profile():
+# what the phase kernel's code is made of: the visit, its ranking and packed operations,
+# the coordinate step, and the choice of its form
+PHASE_SOURCES = ("phase_reg_impl.cuh", "phase_rank.cuh", "packed.cuh", "csc_internal.cuh",
+                 "kernel_phase_reg.cu")
+
+
+def phase_sources_hash(root=ROOT):
+    """16 hex digits over the contents of PHASE_SOURCES (OSError if one is missing)."""
+    import hashlib
+    h = hashlib.sha256()
+    for name in PHASE_SOURCES:
+        with open(os.path.join(root, "paper_1705_10087_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
+def phase_profile(root=ROOT):
     """Per-launch counters of the phase kernel from the committed ncu summary
     (dram_bytes_per_launch, l2_bytes_per_launch, l2_throughput_pct), or {}
-    when the kernel source changed since those counters were taken."""
-    import hashlib
+    when one of PHASE_SOURCES changed since those counters were taken."""
     try:
-        text = open(os.path.join(ROOT, "profiles", f"phase_kernel_{WORKLOAD}.md")).read()
-        src = open(os.path.join(ROOT, "paper_1705_10087_gb300", "csrc",
-                                "phase_reg_impl.cuh"), "rb").read()
+        with open(os.path.join(root, "profiles", f"phase_kernel_{WORKLOAD}.md")) as f:
+            text = f.read()
+        want = phase_sources_hash(root)
     except OSError:
         return {}
     fields = dict(ln.split(":", 1) for ln in text.splitlines()
                   if ln.startswith(("kernel_source", "dram_", "l2_")))
-    if fields.get("kernel_source_sha256_16", "").strip() != hashlib.sha256(src).hexdigest()[:16]:
+    if fields.get("kernel_source_sha256_16", "").strip() != want:
         return {}
     out = {}
     for k in ("dram_bytes_per_launch", "l2_bytes_per_launch", "l2_throughput_pct"):
@@ -818,7 +833,7 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak if achieved else None,
                      "traffic": prof.get("dram_bytes_per_launch"),
-                     "kernel": "phase_kernel", "peak_kind": peak_kind,
+                     "kernel": "phase_reg_kernel", "peak_kind": peak_kind,
                      "avg_launch_us": 1e3 * phase_ms / phase_launches if phase_launches else None,
                      "launches": phase_launches,
                      # the state lives in L2: the level the data are served from
