@@ -964,7 +964,7 @@ struct Block2 {
     void *dev = nullptr;
     size_t cap = 0;
     int device = 0;
-    unsigned long long ctx = 0;  // id of its context (0: unknown)
+    unsigned long long ctx = 0;  // id of its context, a primary one (0: not kept)
     unsigned long long *pin = nullptr;
 };
 struct Kept2 {
@@ -1100,6 +1100,8 @@ cudaError_t take_block2(int device, size_t bytes, Block2 *out)
     }
     b.device = device;
     b.cap = bytes;
+    if (Primary2(device).id != b.ctx)
+        b.ctx = 0;
     cudaError_t e = csc::device_alloc(&b.dev, bytes);
     if (e != cudaSuccess)
         return e;
@@ -1114,8 +1116,7 @@ cudaError_t take_block2(int device, size_t bytes, Block2 *out)
 
 void keep_block2(const Block2 &b)
 {
-    const Primary2 p(b.device);
-    if (b.cap > kKeep2 || p.id == 0 || p.id != b.ctx) {
+    if (b.cap > kKeep2 || b.ctx == 0) {
         free_block2(b);
         return;
     }
