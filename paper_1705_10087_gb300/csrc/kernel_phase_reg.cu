@@ -53,7 +53,8 @@ bool phase_reg_config(int K, int L, int w_max, PhaseConfig *cfg)
         // two bits of the changed mask are the halo's)
         const int ns = (w_max + cb - 1) / cb;
         const size_t smem = phase_reg_smem(nq, groups, L, w_max);
-        if (groups * cb > 512 || ns > 30 || smem > (size_t)kPhaseRegSmem)
+        if (groups * cb > 512 || ns > 30 || groups * nq * 4 > kRegAtoms ||
+            smem > (size_t)kPhaseRegSmem)
             continue;
         cfg->reg_nq = nq;
         cfg->reg_ns = ns;

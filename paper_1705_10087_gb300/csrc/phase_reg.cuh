@@ -26,7 +26,8 @@ RegKernel phase_reg_nq6(int block, int cb, bool dense);
 RegKernel phase_reg_nq7(int block, int cb, bool dense);
 RegKernel phase_reg_nq8(int block, int cb, bool dense);
 
-constexpr int kPhaseRegSmem = kMaxSmem - 8192;  // dynamic shared memory at most (static: 7 KB)
+constexpr int kPhaseRegSmem = kMaxSmem - 8192;  // dynamic shared memory at most (static: 5 KB)
+constexpr int kRegAtoms = 256;  // atoms of all groups at most, padded to whole groups
 // Shared memory (bytes) per group of atoms: the halo of 2 (L-1) columns, the own
 // columns, and per own column a key and the bits of its listed and unlisted
 // nonzeros.  A column takes NQ | 1 quads (an odd stride: 128-bit accesses without

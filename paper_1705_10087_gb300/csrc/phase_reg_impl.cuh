@@ -52,9 +52,6 @@ namespace csc {
 
 namespace {
 
-constexpr int kRegWarps = 16;  // column warps of a block at most (and one active warp)
-constexpr int kRegAtoms = 32 * kRegWarps;  // padded atoms: at most 16 groups of 8 float4
-
 // Index word of a key (key_index, atoms from bit 17 on): the column's bits.
 constexpr int kKeyShift = 17;
 __device__ __forceinline__ unsigned key_pos(unsigned slot, unsigned c)
@@ -64,7 +61,7 @@ __device__ __forceinline__ unsigned key_pos(unsigned slot, unsigned c)
 
 // One launch of a phase.  drain == 0: block b visits segment phase_list[b];
 // else the blocks drain the queue (see launch_phase_drain).
-// TAIL: the last group of atoms may hold fewer than NQ quads.
+// TAIL: several groups of atoms, the last of which may hold fewer than NQ quads.
 template <int NQ, bool TAIL, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
     phase_reg_kernel(PhaseParams pp, int cb, int drain)
@@ -73,7 +70,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const float kNan = __int_as_float(0x7fffffff);
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ __align__(16) unsigned long long s_key[2][32];
-    __shared__ __align__(16) float s_nrm[kRegAtoms], s_rn[kRegAtoms];
+    constexpr int kAtoms = TAIL ? kRegAtoms : N;  // (without TAIL: one group)
+    __shared__ __align__(16) float s_nrm[kAtoms], s_rn[kAtoms];
     // active list: r, z, index word of the key (flags 0), Z' of the last step
     __shared__ __align__(16) float4 s_act[kActive];
     // objective decrease of the visit, in one order whatever lanes hold the nonzeros:
