@@ -19,8 +19,8 @@ RegKernel reg_kernel(const PhaseConfig &cfg, bool dense)
 // Blocks per SM of the form with more registers (96 a thread).  Launches of no more
 // blocks run it: nothing spills in the chain of updates (K = 25, P = 1, L = 200: T = 7396,
 // 18 segments, 21.3 -> 17.6 ms a solve; T = 93,992, 2.47 -> 2.20 ms).  Launches of more,
-// and those that drain a queue, run the one with more blocks per SM (T = 5,000,000: 26.6 ms
-// with one block per SM, 22.4 with two).
+// and those that drain a queue, run the one with more blocks per SM (T = 5,000,000: 26.7 ms
+// with one block per SM, 21.0 with two).
 int roomy_blocks(int block)
 {
     return block <= 160 ? 4 : block <= 288 ? 2 : 1;

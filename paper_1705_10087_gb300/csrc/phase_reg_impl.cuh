@@ -38,7 +38,7 @@
 //   P=7, K=25, L=64, T=200,000, 1024 segments   722 -> 521 us
 //   P=5, K=18, L=51, T=60,013                   2737 -> 570 us
 //   P=1, K=5, L=16, T=2000, 10 segments         734 -> 275 us
-//   P=1, K=25, L=200, T=5,000,000               26.8 -> 18.6 ms
+//   P=1, K=25, L=200, T=5,000,000               26.8 -> 17.2 ms
 // What bounds it now: 2300 cycles per link with one block on an SM (the L2 round
 // trip of the coefficients 600-700 of them); with five blocks the L1/shared
 // pipe (76% busy).
